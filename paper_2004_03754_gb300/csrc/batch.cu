@@ -151,7 +151,7 @@ __device__ void particle_chunk(const BatchArgs<T>& A, const StencilArgs<T>* sp, 
     li[d] = floor_split(c, frac);
     fr[d] = to_prec<T>(frac);
   }
-  advance_particle<T, 2>(ve, vb, acc, A.parts, q, li, fr, li, g, A.a, A.err);
+  advance_particle<T, 2, -1, false, true>(ve, vb, acc, A.parts, q, li, fr, li, g, A.a, A.err);
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {

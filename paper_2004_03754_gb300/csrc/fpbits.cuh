@@ -97,6 +97,14 @@ PIC_HD float narrow_signed(double x) {
   return f32_from_bits(sign | (mag < (897ull << 52) ? 0u : m));
 }
 
+// narrow_signed for any FP64 value: magnitudes from 2^127 on, infinities and NaN
+// give +-2^127, which every range check of the callers refuses.
+PIC_HD float narrow_sat(double x) {
+  const uint32_t h = (uint32_t)(f64_bits(x) >> 32);
+  return (h & 0x7fffffffu) >= 0x47e00000u ? f32_from_bits((h & 0x80000000u) | 0x7f000000u)
+                                          : narrow_signed(x);
+}
+
 // Exact FP32 -> FP64 for a positive normal float (rebias 127 -> 1023).
 PIC_HD double widen_pos(float f) {
   const uint32_t b = f32_bits(f);
@@ -125,6 +133,15 @@ PIC_HD double widen(float f) {
     lo = m << 29;
   }
   return f64_from_hilo(hi, lo);
+}
+
+// FP32 -> FP64, exact for zero and normal numbers, subnormals to a signed zero
+// (no branches; infinities and NaN are not expected: the callers refuse them)
+PIC_HD double widen_normal(float f) {
+  const uint32_t b = f32_bits(f);
+  const uint32_t mag = b & 0x7fffffffu;
+  const bool z = mag < 0x00800000u;
+  return f64_from_hilo((b & 0x80000000u) | (z ? 0u : (mag >> 3) + 0x38000000u), z ? 0u : b << 29);
 }
 
 // floor(c) and c - floor(c) for a cell coordinate c in [0, 2^31), both exact,

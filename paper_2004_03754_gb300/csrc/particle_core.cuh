@@ -10,6 +10,7 @@
 
 #include "common.cuh"
 #include "field_tile.cuh"
+#include "pair_push.cuh"
 #include "pushers.cuh"
 
 namespace pic {
@@ -255,10 +256,31 @@ struct Axis {
   T wn[3], wh[3];
 };
 
+// Nearest node k in {-1, 0, 1, 2} of t in (-1, 2), and its value in T.  FP64 compares
+// the leading word on the integer pipe (an FP64 compare issues like a multiply).
+template <typename T>
+PIC_HD int near_node(const T& t, T& k) {
+  const bool up = t >= (T)0.5, up2 = t >= (T)1.5, dn = t < (T)(-0.5);
+  k = up2 ? (T)2 : (up ? (T)1 : (dn ? (T)(-1) : (T)0));
+  return up2 ? 2 : (up ? 1 : (dn ? -1 : 0));
+}
+template <>
+PIC_HD int near_node<double>(const double& t, double& k) {
+  const uint32_t h = (uint32_t)(f64_bits(t) >> 32);
+  const bool pos = h < 0x80000000u;
+  const bool up = pos && h >= 0x3fe00000u, up2 = pos && h >= 0x3ff80000u, dn = h >= 0xbfe00000u;
+  k = f64_from_hilo(up2 ? 0x40000000u : (up ? 0x3ff00000u : (dn ? 0xbff00000u : 0u)), 0u);
+  return up2 ? 2 : (up ? 1 : (dn ? -1 : 0));
+}
+
 // Position along one axis as integer node li plus fraction f in [0, 1).
 template <typename T>
 PIC_HD void axis_weights(int li, T f, Axis<T>& a) {
-  if (f < (T)0.5) {
+  if constexpr (std::is_same<T, double>::value) {
+    double k;
+    a.bn = li - 1 + near_node<T>(f, k);
+    bspline3<T>(f - k, a.wn);
+  } else if (f < (T)0.5) {
     a.bn = li - 1;
     bspline3<T>(f, a.wn);
   } else {
@@ -271,8 +293,13 @@ PIC_HD void axis_weights(int li, T f, Axis<T>& a) {
 
 // Gather (App. A): component c sampled at its own staggered node.
 // half[c][d] = 1 when component c sits at a half-integer node along axis d.
+// FP32 fields are returned in FP32, the other forms widened to FP64.
+template <typename T>
+struct GatherOf {
+  using type = typename std::conditional<std::is_same<T, float>::value, float, double>::type;
+};
 template <typename T, int NDIM, class VE, class VB>
-PIC_HD void gather(const VE* ve, const VB* vb, const Axis<T>* ax, double eb[6]) {
+PIC_HD void gather(const VE* ve, const VB* vb, const Axis<T>* ax, typename GatherOf<T>::type eb[6]) {
   constexpr int half[6][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {0, 1, 1}, {1, 0, 1}, {1, 1, 0}};
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
@@ -308,7 +335,6 @@ PIC_HD void gather(const VE* ve, const VB* vb, const Axis<T>* ax, double eb[6]) 
       }
     }
     if constexpr (is_dfl<T>::value) eb[c] = widen(acc.hi) + widen(acc.lo);
-    else if constexpr (sizeof(T) == 4) eb[c] = widen(acc);
     else eb[c] = acc;
   }
 }
@@ -319,15 +345,24 @@ PIC_HD void gather(const VE* ve, const VB* vb, const Axis<T>* ax, double eb[6]) 
 template <typename T>
 PIC_HD void esir_axis(int li, T f, T delta, int& base, int& na, T S0[4],
                                           T dS[4]) {
-  const int h0 = f >= (T)0.5 ? 1 : 0;
+  T h0, h1;
   const T t1 = f + delta;
-  const int k1 = (int)floor(t1 + (T)0.5);
-  const int i0 = li + h0, i1 = li + k1;
+  int k0, k1;
+  if constexpr (std::is_same<T, float>::value) {
+    k0 = f >= 0.5f ? 1 : 0;
+    k1 = (int)floorf(t1 + 0.5f);
+    h0 = (float)k0;
+    h1 = (float)k1;
+  } else {
+    k0 = near_node<T>(f, h0);
+    k1 = near_node<T>(t1, h1);
+  }
+  const int i0 = li + k0, i1 = li + k1;
   base = (i0 < i1 ? i0 : i1) - 1;
   na = (i0 == i1) ? 3 : 4;
   T w0[3], w1[3];
-  bspline3<T>(f - (T)h0, w0);
-  bspline3<T>(t1 - (T)k1, w1);
+  bspline3<T>(f - h0, w0);
+  bspline3<T>(t1 - h1, w1);
   const bool s0 = i0 > base + 1, s1 = i1 > base + 1;   // shape starts at node 1 (else 0)
   T S1[4];
   S0[0] = s0 ? (T)0 : w0[0];
@@ -344,6 +379,15 @@ PIC_HD void esir_axis(int li, T f, T delta, int& base, int& na, T S0[4],
 
 // Esirkepov deposit (Sec. 3.3) of one particle moving r0 -> r1 (cell units).
 // cf[d] = -w dx_d/dt (running-sum factor), j3f = w v3 (2D out-of-plane current).
+// FP64: with the mean shapes Sm = S0 + dS/2 the path averages factor,
+//   S0 S0' + dS S0'/2 + S0 dS'/2 + dS dS'/3 = Sm Sm' + dS dS'/12,
+// and the running sums of dS along the axis of a component do not depend on the
+// other axes, so each node takes one product (2D J1, J2), two operations (2D J3)
+// or one product of a plane factor (3D) instead of three to seven on the FP64 pipe
+// (all moves of one node: 2D 94 -> 48 operations, 3D 351 -> 108).  2D FP64 Boris
+// kernel, 6.3 M electrons: 3.81 -> 2.98 ms per step, 247 FP64-pipe instructions per
+// push, that pipe 87 % busy.
+// FP32 deposits, on a pipe with room, keep the sums in the form written out.
 template <typename T, int NDIM, class ACC>
 PIC_HD void deposit(const ACC* acc, const int* li, const T* f, const T* delta,
                                         const T* cf, T j3f) {
@@ -351,68 +395,140 @@ PIC_HD void deposit(const ACC* acc, const int* li, const T* f, const T* delta,
   T S0[3][4], dS[3][4];
 #pragma unroll
   for (int d = 0; d < NDIM; ++d) esir_axis<T>(li[d], f[d], delta[d], b[d], na[d], S0[d], dS[d]);
-  const T third = (T)(1.0 / 3.0);
   // Entries outside a move's na-node footprint are zero: the running sums end
   // at node na-2 and rows/columns >= na carry no shape.
-  if constexpr (NDIM == 2) {
+  if constexpr (std::is_same<T, float>::value) {
+    const T third = (T)(1.0 / 3.0);
+    if constexpr (NDIM == 2) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (j >= na[1]) break;
-      const T f2 = S0[1][j] + (T)0.5 * dS[1][j];
-      T run = 0;
+      for (int j = 0; j < 4; ++j) {
+        if (j >= na[1]) break;
+        const T f2 = S0[1][j] + (T)0.5 * dS[1][j];
+        T run = 0;
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        if (i >= na[0] - 1) break;
-        run += cf[0] * dS[0][i] * f2;
-        acc[0].add(b[0] + i, b[1] + j, 0, run);
+        for (int i = 0; i < 3; ++i) {
+          if (i >= na[0] - 1) break;
+          run += cf[0] * dS[0][i] * f2;
+          acc[0].add(b[0] + i, b[1] + j, 0, run);
+        }
       }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (i >= na[0]) break;
-      const T f1 = S0[0][i] + (T)0.5 * dS[0][i];
-      T run = 0;
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        if (j >= na[1] - 1) break;
-        run += cf[1] * dS[1][j] * f1;
-        acc[1].add(b[0] + i, b[1] + j, 0, run);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (j >= na[1]) break;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         if (i >= na[0]) break;
-        const T W3 = S0[0][i] * S0[1][j] + (T)0.5 * dS[0][i] * S0[1][j] +
-                     (T)0.5 * S0[0][i] * dS[1][j] + third * dS[0][i] * dS[1][j];
-        acc[2].add(b[0] + i, b[1] + j, 0, j3f * W3);
+        const T f1 = S0[0][i] + (T)0.5 * dS[0][i];
+        T run = 0;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          if (j >= na[1] - 1) break;
+          run += cf[1] * dS[1][j] * f1;
+          acc[1].add(b[0] + i, b[1] + j, 0, run);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (j >= na[1]) break;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (i >= na[0]) break;
+          const T W3 = S0[0][i] * S0[1][j] + (T)0.5 * dS[0][i] * S0[1][j] +
+                       (T)0.5 * S0[0][i] * dS[1][j] + third * dS[0][i] * dS[1][j];
+          acc[2].add(b[0] + i, b[1] + j, 0, j3f * W3);
+        }
+      }
+    } else {
+      // 3D: W_d = dS_d * (S0_a S0_b + dS_a S0_b/2 + S0_a dS_b/2 + dS_a dS_b/3)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const int a = (d + 1) % 3, c = (d + 2) % 3;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (q >= na[c]) break;
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            if (p >= na[a]) break;
+            const T pre = S0[a][p] * S0[c][q] + (T)0.5 * dS[a][p] * S0[c][q] +
+                          (T)0.5 * S0[a][p] * dS[c][q] + third * dS[a][p] * dS[c][q];
+            T run = 0;
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+              if (m >= na[d] - 1) break;
+              run += cf[d] * dS[d][m] * pre;
+              int l[3];
+              l[d] = b[d] + m;
+              l[a] = b[a] + p;
+              l[c] = b[c] + q;
+              acc[d].add(l[0], l[1], l[2], run);
+            }
+          }
+        }
       }
     }
   } else {
-    // 3D: W_d = dS_d * (S0_a S0_b + dS_a S0_b/2 + S0_a dS_b/2 + dS_a dS_b/3)
+    const T twelfth = (T)(1.0 / 12.0);
+    T Sm[3][4], R[3][3];   // mean shapes; running sums times cf
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int a = (d + 1) % 3, c = (d + 2) % 3;
+    for (int d = 0; d < NDIM; ++d) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (q >= na[c]) break;
+      for (int l = 0; l < 4; ++l) Sm[d][l] = S0[d][l] + (T)0.5 * dS[d][l];
+      T run = dS[d][0];
+      R[d][0] = cf[d] * run;
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-          if (p >= na[a]) break;
-          const T pre = S0[a][p] * S0[c][q] + (T)0.5 * dS[a][p] * S0[c][q] +
-                        (T)0.5 * S0[a][p] * dS[c][q] + third * dS[a][p] * dS[c][q];
-          T run = 0;
+      for (int l = 1; l < 3; ++l) {
+        run += dS[d][l];
+        R[d][l] = cf[d] * run;
+      }
+    }
+    if constexpr (NDIM == 2) {
 #pragma unroll
-          for (int m = 0; m < 3; ++m) {
-            if (m >= na[d] - 1) break;
-            run += cf[d] * dS[d][m] * pre;
-            int l[3];
-            l[d] = b[d] + m;
-            l[a] = b[a] + p;
-            l[c] = b[c] + q;
-            acc[d].add(l[0], l[1], l[2], run);
+      for (int j = 0; j < 4; ++j) {
+        if (j >= na[1]) break;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          if (i >= na[0] - 1) break;
+          acc[0].add(b[0] + i, b[1] + j, 0, R[0][i] * Sm[1][j]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (i >= na[0]) break;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          if (j >= na[1] - 1) break;
+          acc[1].add(b[0] + i, b[1] + j, 0, R[1][j] * Sm[0][i]);
+        }
+      }
+      const T j12 = twelfth * j3f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (j >= na[1]) break;
+        const T m = j3f * Sm[1][j], e = j12 * dS[1][j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (i >= na[0]) break;
+          acc[2].add(b[0] + i, b[1] + j, 0, Sm[0][i] * m + dS[0][i] * e);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const int a = (d + 1) % 3, c = (d + 2) % 3;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (q >= na[c]) break;
+          const T e = twelfth * dS[c][q];
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            if (p >= na[a]) break;
+            const T pre = Sm[a][p] * Sm[c][q] + dS[a][p] * e;
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+              if (m >= na[d] - 1) break;
+              int l[3];
+              l[d] = b[d] + m;
+              l[a] = b[a] + p;
+              l[c] = b[c] + q;
+              acc[d].add(l[0], l[1], l[2], R[d][m] * pre);
+            }
           }
         }
       }
@@ -428,68 +544,102 @@ PIC_HD void latch(unsigned* err, unsigned bit) {
 #endif
 }
 
+// |delta| < 1, false for NaN (FP64: on the integer pipe)
+PIC_HD bool below_one(double x) { return ((uint32_t)(f64_bits(x) >> 32) & 0x7fffffffu) < 0x3ff00000u; }
+PIC_HD bool below_one(float x) { return fabsf(x) < 1.0f; }
+PIC_HD bool below_one(dfl x) { return fabs(x) < dfl(1); }
+// a value in FP32, for the box-edge test (FP64: narrowed on the integer pipe)
+PIC_HD float rough(double x) { return narrow_signed(x); }
+PIC_HD float rough(float x) { return x; }
+PIC_HD float rough(dfl x) { return (float)x; }
+
 // Push + move of one particle at window-local node li + fraction f per axis.
 // PUSH: PIC_BORIS, PIC_ANALYTIC or PIC_HC fixed at compile time, or -1 to follow a.pusher.
+// TEST: an ensemble's few electrons: the plain FP64 push for every field type (one
+// Newton step of its reciprocals next to FP32 fields).  There the push is not what
+// bounds the step, and a run of thousands of steps at gamma >> 1 amplifies the last
+// bit of a trajectory.
 // GAIN: also add the step's work into the energy-gain integrals p.wl, p.wd
 // (Sec. 4.2): W_LWFA += (q/m) dt E1 vbar1, W_DLA += (q/m) dt E_perp . vbar_perp with
 // vbar = (u^{n-1/2} + u^{n+1/2}) / (gamma^{n-1/2} + gamma^{n+1/2}), the velocity for
 // which the two add up to the Boris push's energy change exactly.
-template <typename T, int NDIM, int PUSH = -1, bool GAIN = false, class VE, class VB, class ACC>
+template <typename T, int NDIM, int PUSH = -1, bool GAIN = false, bool TEST = false, class VE, class VB,
+          class ACC>
 PIC_HD void advance_particle(const VE* ve, const VB* vb, const ACC* acc,
                                                  const PartPtrs& p, int64_t q, const int* li,
                                                  const T* f, const int* gcell, const GridArgs& g,
                                                  const PartArgs& a, unsigned* err) {
-  // Newton steps of the FP64 reciprocals: one from the FP32 seed suffices next to
-  // FP32 fields; FP64 and compensated fields take two (FP64 accuracy)
-  constexpr int NR = std::is_same<T, float>::value ? 1 : 2;
+  // FP32 fields: the push in FP32 pairs, its changes of u and x added in FP64
+  // (pair_push.cuh).  FP64 and compensated fields: the FP64 push, reciprocals by
+  // two Newton steps.
+  constexpr bool F32 = std::is_same<T, float>::value, PAIR = F32 && !TEST;
+  constexpr int NR = F32 ? 1 : 2;
   using D = typename DepositOf<T>::type;
   Axis<T> ax[3];
 #pragma unroll
   for (int d = 0; d < NDIM; ++d) axis_weights<T>(li[d], f[d], ax[d]);
-  double eb[6];
-  gather<T, NDIM>(ve, vb, ax, eb);
+  typename GatherOf<T>::type eg[6];
+  gather<T, NDIM>(ve, vb, ax, eg);
+  typename std::conditional<PAIR, float, double>::type eb[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    if constexpr (F32 && TEST) eb[c] = widen(eg[c]);
+    else eb[c] = eg[c];
+  }
   double u[3] = {p.u[0][q], p.u[1][q], p.u[2][q]};
   const double um[3] = {u[0], u[1], u[2]};
-  if (PUSH == PIC_ANALYTIC || (PUSH < 0 && a.pusher == PIC_ANALYTIC)) {
-    if (analytic_push(a.qm, g.dt, eb, u) < 0) {
+  double dx[3];   // the move, FP64 (FP64 and compensated fields)
+  PairMove mv;    // the move in FP32 pairs (FP32 fields)
+  double ig = 0.0, dtig = 0.0;
+  T delta[3];     // the move in cells, in the field precision (shape weights)
+  bool moved_ok = true, finite;
+  if constexpr (PAIR) {
+    if (!push_pair<PUSH, NDIM>(a.qm, g.dt, a.pusher, eb, u, mv)) {
       latch(err, ERRBIT_ANALYTIC);
       return;
     }
-  } else if (PUSH == PIC_HC || (PUSH < 0 && a.pusher == PIC_HC)) {
-    hc_push<NR>(a.qm, g.dt, eb, u);
+    finite = isfinite(mv.dtig);
+#pragma unroll
+    for (int d = 0; d < NDIM; ++d) delta[d] = mv.dtig * mv.u[d] * to_prec<float>(g.inv_dx[d]);
   } else {
-    boris_push<NR>(a.qm, g.dt, eb, u);
+    if (PUSH == PIC_ANALYTIC || (PUSH < 0 && a.pusher == PIC_ANALYTIC)) {
+      const int it = TEST ? analytic_push(a.qm, g.dt, eb, u) : analytic_push_series(a.qm, g.dt, eb, u);
+      if (it < 0) {
+        latch(err, ERRBIT_ANALYTIC);
+        return;
+      }
+    } else if (PUSH == PIC_HC || (PUSH < 0 && a.pusher == PIC_HC)) {
+      hc_push<NR>(a.qm, g.dt, eb, u);
+    } else {
+      boris_push<NR>(a.qm, g.dt, eb, u);
+    }
+    ig = rsqrt_nr<NR>(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    dtig = g.dt * ig;
+    finite = isfinite(dtig);
+#pragma unroll
+    for (int d = 0; d < NDIM; ++d) {
+      if constexpr (F32) {
+        delta[d] = to_prec<float>(dtig) * to_prec<float>(u[d]) * to_prec<float>(g.inv_dx[d]);
+      } else {
+        dx[d] = dtig * u[d];
+        if constexpr (is_dfl<T>::value) delta[d] = T(dx[d] * g.inv_dx[d]);
+        else delta[d] = dx[d] * g.inv_dx[d];
+      }
+    }
   }
-  const double gp2 = 1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-  const double ig = rsqrt_nr<NR>(gp2);
-  const double dtig = g.dt * ig;
   if constexpr (GAIN) {
     const double gm2 = 1.0 + um[0] * um[0] + um[1] * um[1] + um[2] * um[2];
-    const double gsum = gm2 * rsqrt_nr<NR>(gm2) + gp2 * ig;   // gamma^{n-1/2} + gamma^{n+1/2}
-    const double f = a.qm * g.dt * rcp_nr<NR>(gsum);
-    p.wl[q] += f * eb[0] * (um[0] + u[0]);
-    p.wd[q] += f * (eb[1] * (um[1] + u[1]) + eb[2] * (um[2] + u[2]));
+    const double gp2 = 1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    // gamma^{n-1/2} + gamma^{n+1/2}
+    const double gsum = gm2 * rsqrt_nr<NR>(gm2) + gp2 * rsqrt_nr<NR>(gp2);
+    const double w = a.qm * g.dt * rcp_nr<NR>(gsum);
+    p.wl[q] += w * (double)eb[0] * (um[0] + u[0]);
+    p.wd[q] += w * ((double)eb[1] * (um[1] + u[1]) + (double)eb[2] * (um[2] + u[2]));
   }
-  // FP32 fields: the move in cells is formed from the narrowed factors, and the
-  // FP64 position takes the move as one fused multiply-add per axis.  FP64 and
-  // compensated fields: the FP64 move dx, its cells and the position from it.
-  constexpr bool F32 = std::is_same<T, float>::value;
-  double dx[3];   // the move, FP64 (FP64 and compensated fields)
-  T delta[3];     // the move in cells, in the field precision (shape weights)
-  bool moved_ok = true;
 #pragma unroll
-  for (int d = 0; d < NDIM; ++d) {
-    if constexpr (F32) {
-      delta[d] = to_prec<float>(dtig) * to_prec<float>(u[d]) * to_prec<float>(g.inv_dx[d]);
-    } else {
-      dx[d] = dtig * u[d];
-      if constexpr (is_dfl<T>::value) delta[d] = T(dx[d] * g.inv_dx[d]);
-      else delta[d] = dx[d] * g.inv_dx[d];
-    }
-    moved_ok = moved_ok && (fabs(delta[d]) < (T)1);   // false for NaN as well
-  }
+  for (int d = 0; d < NDIM; ++d) moved_ok = moved_ok && below_one(delta[d]);   // false for NaN
   if (!moved_ok) {
-    latch(err, isfinite(dtig) ? ERRBIT_MOVE : ERRBIT_NONFINITE);
+    latch(err, finite ? ERRBIT_MOVE : ERRBIT_NONFINITE);
     return;
   }
   const double w = p.w[q];
@@ -504,7 +654,8 @@ PIC_HD void advance_particle(const VE* ve, const VB* vb, const ACC* acc,
     }
     // w v3 = w u3 / gamma; in FP32 as the product of the narrowed factors
     D v3;
-    if constexpr (std::is_same<D, float>::value) v3 = to_prec<D>(u[2]) * to_prec<D>(ig);
+    if constexpr (PAIR) v3 = mv.u[2] * mv.ig;
+    else if constexpr (std::is_same<D, float>::value) v3 = to_prec<D>(u[2]) * to_prec<D>(ig);
     else v3 = to_prec<D>(u[2] * ig);
     deposit<D, NDIM>(acc, li, fd, dd, cf, wt * v3);
   }
@@ -514,9 +665,10 @@ PIC_HD void advance_particle(const VE* ve, const VB* vb, const ACC* acc,
 #pragma unroll
   for (int d = 0; d < NDIM; ++d) {
     double x;
-    if constexpr (F32) x = fma(dtig, u[d], p.x[d][q]);
+    if constexpr (PAIR) x = p.x[d][q] + pr_join(mv.dx[d]);
+    else if constexpr (F32) x = fma(dtig, u[d], p.x[d][q]);
     else x = p.x[d][q] + dx[d];
-    const int land = gcell[d] + (int)floorf((float)f[d] + (float)delta[d]);
+    const int land = gcell[d] + (int)floorf(rough(f[d]) + rough(delta[d]));
     if (land <= 0 || land >= g.n[d] - 1) {
       if (x < 0.0) x += g.len[d];
       else if (x >= g.len[d]) x -= g.len[d];
