@@ -64,15 +64,28 @@ void choose_particle_tiles(pic_ctx* c) {
   const int nd = c->grid.ndim;
   PartTile& t = c->ptile;
   int tgt[3], K = 8;
+  const bool f64 = c->grid.precision == PIC_FP64;
   if (nd == 2) {
     tgt[0] = 32; tgt[1] = 16; tgt[2] = 1;
   } else {
     // 3D (few particles per tile): re-binning every step keeps the guard at 3
-    // cells above and 2 below, so the staged windows (13x13x9 nodes, 73 KB in
-    // FP32 with the fixed-point current) fit 3 CTAs per SM; a sweep on the
-    // 512x128x128 case found this faster than larger tiles or guards
-    tgt[0] = 8; tgt[1] = 8; tgt[2] = 4;
+    // cells above and 2 below
+    tgt[0] = 8; tgt[1] = 8; tgt[2] = f64 ? 8 : 4;
     K = 1;
+  }
+  // Small FP64 grids: tiles of fewer cells, down to 8x4 (8x4x4), until there are two
+  // per SM; a tile's particles run on one SM (64x16 cells with a particle each: 82 us
+  // per step on two 32x16 tiles).  FP32 currents keep their tiles: each tile's sums
+  // are rounded to FP32 where tiles meet.
+  while (f64) {
+    int64_t nt = 1;
+    for (int d = 0; d < nd; ++d) nt *= (c->g.n[d] + tgt[d] - 1) / tgt[d];
+    const int lim[3] = {8, 4, 4};
+    int pick = -1;
+    for (int d = 0; d < nd; ++d)
+      if (tgt[d] > lim[d] && (pick < 0 || tgt[d] / lim[d] > tgt[pick] / lim[pick])) pick = d;
+    if (nt >= 2 * 152 || pick < 0) break;
+    tgt[pick] /= 2;
   }
   for (;;) {
     for (int d = 0; d < 3; ++d) {

@@ -111,6 +111,26 @@ cudaError_t launch_laser_expand(const FieldPtrs<T>& f, const GridArgs& g, const 
                                 const double* bprof, double w0, double x2c, double x3c,
                                 cudaStream_t st);
 
+// Windows of a particle tile along axis d: `t` cells with `lo` nodes below and `hi`
+// above; along x1 widened so that it starts and ends on multiples of A columns (pad:
+// the columns added below).  E and B are staged over a particle's gather (one node
+// below its cell, two above, plus the drift g - 3), the current is accumulated over
+// its deposit (two below, three above).
+struct WindowAxis {
+  int lo, w;   // nodes below the tile, with the padding; width
+};
+__host__ __device__ inline WindowAxis window_axis(int d, int t, int lo, int hi, int A) {
+  const int l = d == 0 ? (lo + A - 1) / A * A : lo;
+  const int w = l + t + hi;
+  return WindowAxis{l, d == 0 ? (w + A - 1) / A * A : w};
+}
+__host__ __device__ inline WindowAxis eb_window(int d, int t, int g) {
+  return window_axis(d, t, g - 2, g - 1, 2);
+}
+__host__ __device__ inline WindowAxis j_window(int d, int t, int g, int V) {
+  return window_axis(d, t, g - 1, g, V);
+}
+
 struct PartTile {
   int t[3];      // tile size in cells
   int g[3];      // guard cells of the staged window

@@ -1,9 +1,9 @@
-// particle_kernels.cuh -- the tiled particle kernel, the time-centred-B row
-// kernel and the straggler kernel of libpic with their launchers, as templates
-// over the field type; particles_f32.cu, particles_f64.cu and particles_dfl.cu
-// instantiate one field type each (parallel compilation).
+// particle_kernels.cuh -- the tiled particle kernel and the straggler kernel of
+// libpic with their launchers, as templates over the field type; particles_f32.cu,
+// particles_f64.cu and particles_dfl.cu instantiate one field type each (parallel
+// compilation).
 //
-// Particles are binned by tile (a box of cells).  A row pass first forms the
+// Particles are binned by tile (a box of cells).  The Faraday pass has formed the
 // time-centred B^n = B^{n-1/2} - (dt/2) d_E x E^n (Eq. (7) in its half-step form)
 // over the grid.  One CTA owns one tile: it stages E^n and B^n of the tile plus
 // a guard in shared memory and runs every particle of the bin through
@@ -19,6 +19,8 @@
 #pragma once
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "field_tile.cuh"
 #include "particle_core.cuh"
@@ -27,33 +29,47 @@ namespace pic {
 
 namespace {
 
-// Visit every row (c, l3, l2), c < 3, l3 < N3, l2 < N2, of a window whose rows
-// hold W1 values, spread over the CTA's warps by nested loops (no integer
-// division per row); rows of at most 16 values go two per warp, 16 lanes each.
-// (3D windows: short rows and few particles per tile, so this bookkeeping
-// would otherwise dominate the tile's instructions.)
-// f(c, l2, l3, sub_lane, lanes_per_row) runs on the lanes of one row.
-template <class F>
-__device__ __forceinline__ void for_window_rows(int N2, int N3, int W1, int lane, int warp,
-                                                int nwarp, F&& f) {
-  const int split = W1 <= 16 ? 2 : 1;
-  const int sw = 32 / split;
-  const int sub = split == 2 ? lane >> 4 : 0, sl = split == 2 ? lane & 15 : lane;
-  const int step = nwarp * split;
-  for (int c = 0; c < 3; ++c)
-    for (int l3 = 0; l3 < N3; ++l3)
-      for (int l2 = warp * split + sub; l2 < N2; l2 += step) f(c, l2, l3, sl, sw);
+// 16-byte (N = 16) or single-value copies into shared memory, in flight until
+// stage_wait
+template <int N>
+__device__ __forceinline__ void stage_copy(void* dst, const void* src) {
+  if constexpr (N == 16)   // (8 bytes: two FP32 columns)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)), "l"(src), "n"(N) : "memory");
+}
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The rows (l2, l3) of a window in chunks: f(o, j, k, c) for every chunk -- o its
+// offset in a component of the window, (j, k) its x2, x3 grid indices, c its x1 grid
+// column -- spread over the CTA's threads.  A chunk is C values (16 bytes, or one
+// value where grid rows don't start on 16-byte boundaries); the thread's chunk
+// advances by the same step each time, so no division runs in the loop but the one
+// by W2 (3D).  All three components share the index arithmetic.
+template <int C, int NDIM, class F>
+__device__ __forceinline__ void for_window_chunks(const int* W, const int* wlo, const GridArgs& g,
+                                                  F&& f) {
+  const int cpr = W[0] / C, rows = W[1] * W[2];
+  const int dr = (int)blockDim.x / cpr, dc = (int)blockDim.x - dr * cpr;
+  int row = (int)threadIdx.x / cpr, ch = (int)threadIdx.x - row * cpr;
+  while (row < rows) {
+    const int l3 = NDIM == 3 ? row / W[1] : 0, l2 = NDIM == 3 ? row - l3 * W[1] : row;
+    f(row * W[0] + ch * C, pwrap(wlo[1] + l2, g.n[1]), NDIM == 3 ? pwrap(wlo[2] + l3, g.n[2]) : 0,
+      pwrap(wlo[0] + ch * C, g.n[0]));
+    row += dr;
+    ch += dc;
+    if (ch >= cpr) {
+      ch -= cpr;
+      ++row;
+    }
+  }
 }
 
-// W values of a periodic row from column g0, lanes sl of sw per row
-template <typename T>
-__device__ __forceinline__ void stage_row_lanes(T* dst, const T* src, int g0, int W, int n1, int sl,
-                                                int sw) {
-  if (g0 >= 0 && g0 + W <= n1) {
-    for (int l1 = sl; l1 < W; l1 += sw) dst[l1] = src[g0 + l1];
-  } else {
-    for (int l1 = sl; l1 < W; l1 += sw) dst[l1] = src[pwrap(g0 + l1, n1)];
-  }
+// p[0..3] += v[0..3], one 16-byte reduction
+__device__ __forceinline__ void red_add4(float* p, const float* v) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3])
+               : "memory");
 }
 
 // threads 0 .. NDIM+3 ask L2 for one particle array each over [c0, c1) (bulk
@@ -72,57 +88,89 @@ __device__ __forceinline__ void prefetch_chunk(const PartPtrs& p, int64_t c0, in
                "r"((unsigned)((e0 - s0) * 8)) : "memory");
 }
 
-// The time-centred B^n is read from a global array formed once per step by
-// bbar_rows_kernel; E^n and B^n are staged over the particle window, the
-// current is accumulated in a shared-memory window (in int32 fixed point,
-// FixAcc / FixAcc64) and added into the global current once.
-// All staging and the current flush run row by row, one warp per row.
-// PUSH: the pusher, fixed per instance so that the 2D mixed-precision Boris
-// kernel is not held to the analytic pusher's register budget: it fits in 64
-// registers and runs 4 CTAs per SM instead of 3.  8-byte fields: the windows
-// fit 2 (2D) or 1 (3D) CTAs per SM, so the register budget follows.
+// Threads per CTA and CTAs per SM of the tile kernel, with the tile shapes of
+// choose_particle_tiles.  Measured: 3D FP32, 84 M electrons, two steps and their
+// read-back, 2 x 512 threads 38.7 ms (a thread per particle of a tile at 2 per cell;
+// 2 x 256 40.2, 3 x 256 41.1, 2 x 384 44.0, 1 x 512 43.8); 3D FP64, four steps on
+// 301x60x44, one CTA of 384 on 8x8x8 cells 11.6 ms (512 threads 11.8, 2 x 256 on
+// 8x8x4 12.0); 2D FP32, ten Boris steps of 29 M electrons, 3 x 256 at 80 registers
+// 18.2 ms (4 x 256 at 64, which spill, 19.2; 2 x 256 20.4; 1 x 512 21.6).
+template <typename T, int NDIM>
+struct TileCfg {
+  static constexpr bool F = sizeof(T) == 4;
+  static constexpr int threads = NDIM == 3 ? (F ? 512 : 384) : 256;
+  static constexpr int ctas = NDIM == 3 ? (F ? 2 : 1) : (F ? 3 : 2);
+};
+
+// The time-centred B^n is read from a global array formed once per step; E^n and
+// B^n are staged over the particle window by asynchronous 16-byte copies, the
+// current is accumulated in a shared-memory window (in int32 fixed point, FixAcc /
+// FixAcc64) and added into the global current once, 16 bytes at a time for FP32.
+// In 3D a tile holds few particles per window node (512 particles at 2 per cell, 924
+// nodes of E, B and 1872 of the current), so the window's handling counts as much as
+// the particles': copied and flushed value by value it took half the kernel's
+// instructions (84 M electrons, two steps and their read-back 62.8 -> 38.7 ms; 2D,
+// 29 M electrons, ten steps 23.7 -> 19.1 ms).
 template <typename T, int NDIM, int PUSH, bool GAIN>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? ((PUSH == PIC_BORIS && NDIM == 2) ? 4 : 3)
-                                                      : (NDIM == 2 ? 2 : 1))
+__global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::ctas)
     particle_kernel(FieldPtrs<T> f, BbarPtrs<T> bg, PartPtrs p, GridArgs g, StencilArgs<T> s,
                     PartTile t, PartArgs a, BinBufs bins) {
   using D = typename DepositOf<T>::type;
+  constexpr int V = VecOf<T>::V;
   // current window: FP32 deposits as two int32 fixed-point sums (FixAcc), FP64
   // deposits as three (FixAcc64)
   constexpr bool F64 = std::is_same<D, double>::value;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long wmax_warp[32];
   T* sm = reinterpret_cast<T*>(smem_raw);
-  const int64_t tile = blockIdx.x;
+  const unsigned tile = blockIdx.x;
   const int64_t pbeg = bins.start[tile], pend = bins.start[tile + 1];
   if (pbeg == pend) return;
   prefetch_chunk<NDIM>(p, pbeg, min(pend, pbeg + (int64_t)blockDim.x));
   int tc[3];
   {
-    int64_t r = tile;
-    tc[0] = (int)(r % t.nt[0]);
-    r /= t.nt[0];
-    tc[1] = (int)(r % t.nt[1]);
-    tc[2] = (int)(r / t.nt[1]);
+    const unsigned r = tile / (unsigned)t.nt[0];
+    tc[0] = (int)(tile - r * (unsigned)t.nt[0]);
+    tc[2] = NDIM == 3 ? (int)(r / (unsigned)t.nt[1]) : 0;
+    tc[1] = (int)(r - (unsigned)tc[2] * (unsigned)t.nt[1]);
   }
-  const int n1 = g.n[0], n2 = g.n[1], n3 = (NDIM == 3) ? g.n[2] : 1;
+  const int n1 = g.n[0], n2 = g.n[1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  // window: the tile plus g - 1 guard cells below and g above (a particle's
-  // gather and deposit reach two nodes below its cell and three above; g - 3
-  // cells of drift are allowed on both sides)
-  int W[3], wlo[3];
+  // two windows (common.cuh): E, B over the particles' gather, the current over
+  // their deposit; g - 3 cells of drift are allowed on both sides
+  int We[3], elo[3], W[3], wlo[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    W[d] = (d < NDIM) ? t.t[d] + 2 * t.g[d] - 1 : 1;
-    wlo[d] = (d < NDIM) ? tc[d] * t.t[d] - (t.g[d] - 1) : 0;
+    const WindowAxis ew = d < NDIM ? eb_window(d, t.t[d], t.g[d]) : WindowAxis{0, 1};
+    const WindowAxis jw = d < NDIM ? j_window(d, t.t[d], t.g[d], V) : WindowAxis{0, 1};
+    We[d] = ew.w;
+    W[d] = jw.w;
+    elo[d] = d < NDIM ? tc[d] * t.t[d] - ew.lo : 0;
+    wlo[d] = d < NDIM ? tc[d] * t.t[d] - jw.lo : 0;
   }
-  const int nW = W[0] * W[1] * W[2];
-  T* sE = sm;                 // [3][W3][W2][W1]
-  T* sB = sE + 3 * nW;        // [3][W3][W2][W1], the time-centred B
-  int* sJh = reinterpret_cast<int*>(sB + 3 * nW);   // current: [3][W3][W2][W1] per limb, hi first
-  int* sJl = sJh + 3 * nW;
-  int* sJc = sJl + 3 * nW;                          // FP64: the third limb
+  const int nE = We[0] * We[1] * We[2], nW = W[0] * W[1] * W[2];
+  T* sE = sm;                 // [3][We3][We2][We1]
+  T* sB = sE + 3 * nE;        // [3][We3][We2][We1], the time-centred B
+  int* sJh = reinterpret_cast<int*>(smem_raw + ((size_t)nE * 6 * sizeof(T) + 15) / 16 * 16);
+  int* sJl = sJh + 3 * nW;    // current: [3][W3][W2][W1] per limb, hi first
+  int* sJc = sJl + 3 * nW;    // FP64: the third limb
+  // rows on 2-column and on 16-byte boundaries
+  const bool pairs = (n1 & 1) == 0, vec = n1 % V == 0;
 
+  auto stage = [&](auto C) {
+    constexpr int c = decltype(C)::value;
+    for_window_chunks<c, NDIM>(We, elo, g, [&](int o, int j, int k, int i) {
+      const int64_t r = ((int64_t)k * n2 + j) * n1 + i;
+      stage_copy<c * (int)sizeof(T)>(sE + o, f.e[0] + r);
+      stage_copy<c * (int)sizeof(T)>(sE + nE + o, f.e[1] + r);
+      stage_copy<c * (int)sizeof(T)>(sE + 2 * nE + o, f.e[2] + r);
+      stage_copy<c * (int)sizeof(T)>(sB + o, bg.b[0] + r);
+      stage_copy<c * (int)sizeof(T)>(sB + nE + o, bg.b[1] + r);
+      stage_copy<c * (int)sizeof(T)>(sB + 2 * nE + o, bg.b[2] + r);
+    });
+  };
+  if (pairs) stage(std::integral_constant<int, 2>{});
+  else stage(std::integral_constant<int, 1>{});
   {
     // largest |w| of the tile (non-negative doubles order as their bit patterns)
     unsigned long long wm = 0ull;
@@ -132,27 +180,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? ((PUSH == PIC_BORIS && N
     for (int o = 16; o > 0; o >>= 1) wm = max(wm, __shfl_xor_sync(0xffffffffu, wm, o));
     if (lane == 0) wmax_warp[warp] = wm;
   }
-  if constexpr (NDIM == 3) {
-    // short rows: division-free row loops, two rows per warp
-    for_window_rows(W[1], W[2], W[0], lane, warp, nwarp, [&](int c, int l2, int l3, int sl, int sw) {
-      const int gj = pwrap(wlo[1] + l2, n2);
-      const int gk = pwrap(wlo[2] + l3, n3);
-      const int64_t r = ((int64_t)gk * n2 + gj) * n1;
-      const int o = ((c * W[2] + l3) * W[1] + l2) * W[0];
-      const T* e = c == 0 ? f.e[0] : (c == 1 ? f.e[1] : f.e[2]);
-      const T* b = c == 0 ? bg.b[0] : (c == 1 ? bg.b[1] : bg.b[2]);
-      stage_row_lanes(sE + o, e + r, wlo[0], W[0], n1, sl, sw);
-      stage_row_lanes(sB + o, b + r, wlo[0], W[0], n1, sl, sw);
-    });
-  } else {
-    for (int row = warp; row < 3 * W[1]; row += nwarp) {
-      const int l2 = row % W[1], c = row / W[1];
-      const int64_t r = (int64_t)pwrap(wlo[1] + l2, n2) * n1;
-      stage_row<false>(sE + row * W[0], f.e[c] + r, wlo[0], W[0], n1, lane);
-      stage_row<false>(sB + row * W[0], bg.b[c] + r, wlo[0], W[0], n1, lane);
-    }
+  // (the width is a multiple of V, so the limbs are whole 8- or 16-byte words)
+  for (int q = threadIdx.x * 4; q < (F64 ? 9 : 6) * nW; q += blockDim.x * 4) {
+    if (q + 4 <= (F64 ? 9 : 6) * nW) *reinterpret_cast<int4*>(sJh + q) = make_int4(0, 0, 0, 0);
+    else *reinterpret_cast<int2*>(sJh + q) = make_int2(0, 0);
   }
-  for (int q = threadIdx.x; q < (F64 ? 9 : 6) * nW; q += blockDim.x) sJh[q] = 0;
+  stage_wait();
   __syncthreads();
   float S = 1.0f, L = 1.0f;
   int eS = 0, l64 = 0;
@@ -168,11 +201,13 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? ((PUSH == PIC_BORIS && N
     else fix_scales(pend - pbeg, narrow_signed(__longlong_as_double((long long)wm)) * 1.001f, S, L);
   }
 
+  // views indexed by the current window's node
   SmemView<T> ve[3], vb[3];
+  const int eoff = ((elo[2] - wlo[2]) * We[1] + (elo[1] - wlo[1])) * We[0] + (elo[0] - wlo[0]);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    ve[c] = SmemView<T>{sE + c * nW, W[0], W[0] * W[1], 0};
-    vb[c] = SmemView<T>{sB + c * nW, W[0], W[0] * W[1], 0};
+    ve[c] = SmemView<T>{sE + c * nE - eoff, We[0], We[0] * We[1], 0};
+    vb[c] = SmemView<T>{sB + c * nE - eoff, We[0], We[0] * We[1], 0};
   }
   using Acc = typename std::conditional<F64, FixAcc64, FixAcc>::type;
   Acc acc[3];
@@ -192,10 +227,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? ((PUSH == PIC_BORIS && N
     if constexpr (F64) return fix64_decode(sJh[c * nW + q], sJl[c * nW + q], sJc[c * nW + q], i0, i1, i2);
     else return fix_decode(sJh[c * nW + q], sJl[c * nW + q], invS, invSL);
   };
-  int ulo[3], uhi[3];   // periodic unwrap limits of the window-local node index
+  // window-local cell index: periodic unwrap limits [ulo, uhi) (the grid's period
+  // centred on the tile with its drift) and the cells a particle may be in
+  int ulo[3], uhi[3], lmin[3], lmax[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    ulo[d] = (W[d] - g.n[d]) / 2;
+    const int tile0 = d < NDIM ? tc[d] * t.t[d] - wlo[d] : 0, dr = d < NDIM ? t.g[d] - 3 : 0;
+    lmin[d] = tile0 - dr;
+    lmax[d] = tile0 + (d < NDIM ? t.t[d] : 1) - 1 + dr;
+    ulo[d] = lmin[d] + (lmax[d] - lmin[d] + 1 - g.n[d]) / 2;
     uhi[d] = ulo[d] + g.n[d];
   }
   for (int64_t q = pbeg + threadIdx.x; q < pend; q += blockDim.x) {
@@ -216,7 +256,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? ((PUSH == PIC_BORIS && N
       if (l < ulo[d]) l += g.n[d];
       else if (l >= uhi[d]) l -= g.n[d];
       li[d] = l;
-      inside = inside && l >= 2 && l <= W[d] - 4;
+      inside = inside && l >= lmin[d] && l <= lmax[d];
     }
     if (!inside) {
       const unsigned long long slot = atomicAdd(bins.strag_count, 1ull);
@@ -226,28 +266,53 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? ((PUSH == PIC_BORIS && N
     advance_particle<T, NDIM, PUSH, GAIN>(ve, vb, acc, p, q, li, fr, gc, g, a, bins.err);
   }
   __syncthreads();
-  if constexpr (NDIM == 3) {
-    for_window_rows(W[1], W[2], W[0], lane, warp, nwarp, [&](int c, int l2, int l3, int sl, int sw) {
-      const int gj = pwrap(wlo[1] + l2, n2);
-      const int gk = pwrap(wlo[2] + l3, n3);
-      T* dst = (c == 0 ? f.j[0] : (c == 1 ? f.j[1] : f.j[2])) + ((int64_t)gk * n2 + gj) * n1;
-      const int o = (l3 * W[1] + l2) * W[0];
-      const bool inrow = wlo[0] >= 0 && wlo[0] + W[0] <= n1;
-      for (int l1 = sl; l1 < W[0]; l1 += sw) {
-        const D v = jval(c, o + l1);
-        if (v != (D)0) atomic_acc(dst + (inrow ? wlo[0] + l1 : pwrap(wlo[0] + l1, n1)), v);
+  auto flush = [&](auto C) {
+    constexpr int c = decltype(C)::value;
+    for_window_chunks<c, NDIM>(W, wlo, g, [&](int o, int j, int k, int i) {
+      const int64_t r = ((int64_t)k * n2 + j) * n1 + i;
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        T* dst = (m == 0 ? f.j[0] : (m == 1 ? f.j[1] : f.j[2])) + r;
+        D v[c];
+        bool any = false;
+#pragma unroll
+        for (int e = 0; e < c; ++e) {
+          v[e] = jval(m, o + e);
+          any = any || v[e] != (D)0;
+        }
+        if (!any) continue;
+        if constexpr (c == 4 && std::is_same<T, float>::value) {
+          red_add4(dst, v);
+        } else {
+#pragma unroll
+          for (int e = 0; e < c; ++e)
+            if (v[e] != (D)0) atomic_acc(dst + e, v[e]);
+        }
       }
     });
-  } else {
-    for (int row = warp; row < 3 * W[1]; row += nwarp) {
-      const int l2 = row % W[1], c = row / W[1];
-      const int gj = pwrap(wlo[1] + l2, n2);
-      T* dst = f.j[c] + (int64_t)gj * n1;
-      for (int l1 = lane; l1 < W[0]; l1 += 32) {
-        const D v = jval(c, l2 * W[0] + l1);
-        if (v != (D)0) atomic_acc(dst + pwrap(wlo[0] + l1, n1), v);
+  };
+  const int n3 = NDIM == 3 ? g.n[2] : 1;
+  if (W[0] > n1 || W[1] > n2 || W[2] > n3) {
+    // the window wraps onto itself: one thread per grid node sums its window nodes,
+    // in a fixed order
+    const int m0 = min(W[0], n1), m1 = min(W[1], n2), m2 = min(W[2], n3);
+    for (int q = threadIdx.x; q < m0 * m1 * m2; q += blockDim.x) {
+      const int r = q / m0, i0 = q - r * m0, k0 = r / m1, j0 = r - k0 * m1;
+      const int64_t o = ((int64_t)pwrap(wlo[2] + k0, n3) * n2 + pwrap(wlo[1] + j0, n2)) * n1 +
+                        pwrap(wlo[0] + i0, n1);
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        D v = 0;
+        for (int k = k0; k < W[2]; k += n3)
+          for (int j = j0; j < W[1]; j += n2)
+            for (int i = i0; i < W[0]; i += n1) v += jval(m, (k * W[1] + j) * W[0] + i);
+        if (v != (D)0) atomic_acc((m == 0 ? f.j[0] : (m == 1 ? f.j[1] : f.j[2])) + o, v);
       }
     }
+  } else if (vec) {
+    flush(std::integral_constant<int, V>{});
+  } else {
+    flush(std::integral_constant<int, 1>{});
   }
 }
 
@@ -371,7 +436,7 @@ cudaError_t launch_bbar_rows_mt(const FieldPtrs<T>& f, const BbarPtrs<T>& bg, co
 }
 
 // Particles that left their tile's window: the whole update through global
-// memory, with the time-centred B from bg (formed by the tile step's launcher).
+// memory, with the time-centred B from bg.
 template <typename T, int NDIM, bool GAIN>
 __global__ void straggler_kernel(FieldPtrs<T> f, BbarPtrs<T> bg, PartPtrs p, GridArgs g,
                                  StencilArgs<T> s, PartArgs a, BinBufs bins) {
@@ -408,10 +473,10 @@ __global__ void straggler_kernel(FieldPtrs<T> f, BbarPtrs<T> bg, PartPtrs p, Gri
 template <typename T, class K>
 cudaError_t launch_tiles(K kern, const FieldPtrs<T>& f, const BbarPtrs<T>& bg, const PartPtrs& p,
                          const GridArgs& g, const StencilArgs<T>& s, const PartTile& t,
-                         const PartArgs& a, const BinBufs& b, size_t smem, cudaStream_t st) {
+                         const PartArgs& a, const BinBufs& b, size_t smem, int threads, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)t.ntiles, 256, smem, st>>>(f, bg, p, g, s, t, a, b);
+  kern<<<(unsigned)t.ntiles, threads, smem, st>>>(f, bg, p, g, s, t, a, b);
   return cudaGetLastError();
 }
 
@@ -420,12 +485,15 @@ template <typename T, int NDIM, bool GAIN>
 cudaError_t launch_pushers(const FieldPtrs<T>& f, const BbarPtrs<T>& bg, const PartPtrs& p,
                            const GridArgs& g, const StencilArgs<T>& s, const PartTile& t,
                            const PartArgs& a, const BinBufs& b, size_t smem, cudaStream_t st) {
+  constexpr int threads = TileCfg<T, NDIM>::threads;
   if (a.pusher == PIC_ANALYTIC)
     return launch_tiles(particle_kernel<T, NDIM, PIC_ANALYTIC, GAIN>, f, bg, p, g, s, t, a, b, smem,
-                        st);
+                        threads, st);
   if (a.pusher == PIC_HC)
-    return launch_tiles(particle_kernel<T, NDIM, PIC_HC, GAIN>, f, bg, p, g, s, t, a, b, smem, st);
-  return launch_tiles(particle_kernel<T, NDIM, PIC_BORIS, GAIN>, f, bg, p, g, s, t, a, b, smem, st);
+    return launch_tiles(particle_kernel<T, NDIM, PIC_HC, GAIN>, f, bg, p, g, s, t, a, b, smem,
+                        threads, st);
+  return launch_tiles(particle_kernel<T, NDIM, PIC_BORIS, GAIN>, f, bg, p, g, s, t, a, b, smem,
+                      threads, st);
 }
 
 template <typename T>

@@ -175,14 +175,17 @@ inline int grid_for(int64_t n) {
 
 size_t particle_smem_bytes(int ndim, size_t tsize, const PartTile& t, int M) {
   (void)M;
-  // the window: tile + (g - 1) guard cells below and g above, per axis
-  size_t W1 = t.t[0] + 2 * t.g[0] - 1, W2 = t.t[1] + 2 * t.g[1] - 1,
-         W3 = ndim == 3 ? t.t[2] + 2 * t.g[2] - 1 : 1;
-  // E^n and the time-centred B over the window in the field precision; the current
-  // per node: two int32 fixed-point sums per component for an FP32 deposit (24
-  // bytes), three for FP64 (36 bytes; for 8-byte fields both forms fit in it)
+  const int V = 16 / (int)tsize;
+  size_t ne = 1, nj = 1;   // nodes of the E, B window and of the current's
+  for (int d = 0; d < ndim; ++d) {
+    ne *= eb_window(d, t.t[d], t.g[d]).w;
+    nj *= j_window(d, t.t[d], t.g[d], V).w;
+  }
+  // E^n and the time-centred B in the field precision; the current per node: two
+  // int32 fixed-point sums per component for an FP32 deposit (24 bytes), three for
+  // FP64 (36 bytes; for 8-byte fields both forms fit in it)
   const size_t jb = tsize == 8 ? 36 : 24;
-  return W1 * W2 * W3 * (6 * tsize + jb);
+  return (ne * 6 * tsize + 15) / 16 * 16 + nj * jb;
 }
 
 cudaError_t launch_bin_count(const PartPtrs& p, const GridArgs& g, const PartTile& t,
