@@ -107,6 +107,12 @@ void choose_particle_tiles(pic_ctx* c) {
     if (cfl > 0) Kmax = std::min(Kmax, 1 + (int)floor((t.g[d] - 3) / cfl + 1e-12));
   }
   c->sort_interval = std::max(1, Kmax);
+  // a particle moves less than dt/dx cells per step (the margin covers the rounding of
+  // gamma): until this many steps after a re-binning none can have left its window
+  int safe = 1 << 20;
+  for (int d = 0; d < nd; ++d)
+    safe = std::min(safe, (int)floor((t.g[d] - 3) / (c->dt * c->g.inv_dx[d] * (1 + 1e-6))));
+  c->straggle_after = safe;
   t.ntiles = 1;
   for (int d = 0; d < 3; ++d) {
     t.nt[d] = d < nd ? (c->g.n[d] + t.t[d] - 1) / t.t[d] : 1;
@@ -236,39 +242,72 @@ pic_status rebin(pic_ctx* c) {
   return PIC_OK;
 }
 
+// Whether the field step runs as one fused kernel (fields.cu) rather than as a
+// Faraday and an Ampere pass (field_halves.cu): when the caller chose its shape, and
+// for large 2D FP32 vacuum grids whose rows the warps can stream, where the 15 values
+// of HBM traffic per cell decide.  With particles the Faraday pass is needed anyway
+// (it forms the time-centred B).  Measured per step in vacuum, passes against fused:
+// FP32 2048x512 16.4 / 19.3 us, 2048x1024 27.9 / 30.5, 4096x1024 63.8 / 50.9,
+// 512x128x128 116 / 164; FP64 512x128 25.5 / 70.0, 4096x1024 1174 / 1457, 512x128x128
+// 2450 / 3982; compensated 4096x1024 245 / 763, 512x128x128 558 / 976.
+constexpr int64_t kFusedMinCells = 3 << 20;
+
+template <typename T>
+bool field_step_fused(const pic_ctx* c) {
+  if (c->ftile_set) return true;
+  if (c->np > 0 || c->grid.ndim != 2 || !std::is_same<T, float>::value) return false;
+  const Reach R(stencil_mt(c->M), VecOf<T>::V);
+  return c->g.n[0] % VecOf<T>::V == 0 && R.WE(c->ftile.sw, VecOf<T>::V) <= c->g.n[0] &&
+         c->g.ncell >= kFusedMinCells;
+}
+
 template <typename T>
 pic_status one_step(pic_ctx* c, const StencilArgs<T>& s) {
   if (c->steps_since_sort >= c->sort_interval) {
     pic_status st = rebin(c);
     if (st != PIC_OK) return st;
   }
-  for (int k = 0; k < 3; ++k) CK(c, cudaMemsetAsync(c->fj[k], 0, c->tsize * c->g.ncell, c->stream));
-  FieldPtrs<T> f = fields<T>(c, c->cur);
-  if (c->np > 0) {
-    CK(c, cudaMemsetAsync(c->bins.strag_count, 0, sizeof(unsigned long long), c->stream));
+  FieldPtrs<T> f = fields<T>(c, c->cur), o = fields<T>(c, 1 - c->cur);
+  BbarPtrs<T> bg{{(T*)c->bbar[0], (T*)c->bbar[1], (T*)c->bbar[2]}};
+  const bool parts = c->np > 0;
+  if (!parts && !c->j_zero)
+    for (int k = 0; k < 3; ++k)
+      CK(c, cudaMemsetAsync(c->fj[k], 0, c->tsize * c->g.ncell, c->stream));
+  c->j_zero = !parts;
+  const bool fused = field_step_fused<T>(c);
+  // with particles the Faraday pass comes first (it forms the time-centred B that
+  // they see and clears the current); its B^{n+1/2} is written once more by a fused
+  // kernel chosen by the caller
+  if (parts || !fused) {
+    TimedScope ts(c, 4, 1);
+    CK(c, launch_faraday<T>(f, o, parts ? &bg : nullptr, c->g, s, c->bins.strag_count, c->stream));
+  }
+  if (parts) {
     PartArgs a{c->qm, c->grid.pusher, c->np};
     {
-      TimedScope ts(c, 1, c->grid.ndim == 3 ? 2 : 1);
-      BbarPtrs<T> bg{{(T*)c->bbar[0], (T*)c->bbar[1], (T*)c->bbar[2]}};
+      TimedScope ts(c, 1, 1);
       CK(c, launch_particle_step<T>(f, bg, c->parts[c->pcur], c->g, s, c->ptile, a, c->bins,
                                     c->stream));
     }
-    {
+    if (c->steps_since_sort > c->straggle_after || c->strag_always) {
       TimedScope ts(c, 2, 1);
-      BbarPtrs<T> bg{{(T*)c->bbar[0], (T*)c->bbar[1], (T*)c->bbar[2]}};
       CK(c, launch_straggler_step<T>(f, bg, c->parts[c->pcur], c->g, s, a, c->bins, c->np,
                                      c->stream));
     }
+    if (c->corr) {
+      TimedScope ts(c, 3, 1);
+      CK(c, launch_correct_j1<T>((T*)c->fj[0], (T*)c->jtmp, c->g, (const T*)c->taps, c->taps_lo,
+                                 c->taps_n, c->corr_path, c->stream));
+    }
   }
-  if (c->corr) {
-    TimedScope ts(c, 3, 1);
-    CK(c, launch_correct_j1<T>((T*)c->fj[0], (T*)c->jtmp, c->g, (const T*)c->taps, c->taps_lo,
-                               c->taps_n, c->corr_path, c->stream));
-  }
-  FieldPtrs<T> o = fields<T>(c, 1 - c->cur);
   {
     TimedScope ts(c, 4, 1);
-    CK(c, launch_field_step<T>(f, o, c->g, s, c->ftile, c->bins.err, c->stream));
+    if (fused) {
+      CK(c, launch_field_step<T>(f, o, c->g, s, c->ftile, c->bins.err, c->stream));
+    } else {
+      if (!parts) f.j[0] = f.j[1] = f.j[2] = nullptr;
+      CK(c, launch_ampere<T>(f, o, c->g, s, c->stream));
+    }
   }
   if (c->timing) c->t_steps++;
   c->cur = 1 - c->cur;
@@ -506,6 +545,7 @@ pic_status pic_init(const pic_grid* grid, double dt, const pic_coeffs* coeffs, v
     return init_fail(PIC_ERR_OOM);
   }
   cudaMemsetAsync(c->bins.err, 0, sizeof(unsigned), c->stream);
+  cudaMemsetAsync(c->bins.strag_count, 0, sizeof(unsigned long long), c->stream);
   cudaMemsetAsync(c->bins.start, 0, sizeof(int64_t) * (c->ptile.ntiles + 2), c->stream);
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
@@ -703,6 +743,7 @@ pic_status one_step_spectral(pic_ctx* c) {
     if (st != PIC_OK) return st;
   }
   for (int k = 0; k < 3; ++k) CK(c, cudaMemsetAsync(c->fj[k], 0, c->tsize * c->g.ncell, c->stream));
+  c->j_zero = c->np == 0;
   FieldPtrs<double> f = fields<double>(c, c->cur);
   FieldPtrs<double> o = fields<double>(c, 1 - c->cur);
   double* bb[3] = {(double*)c->bbar[0], (double*)c->bbar[1], (double*)c->bbar[2]};
@@ -713,7 +754,6 @@ pic_status one_step_spectral(pic_ctx* c) {
   if (c->np > 0) {
     CK(c, cudaMemsetAsync(c->bins.strag_count, 0, sizeof(unsigned long long), c->stream));
     PartArgs a{c->qm, c->grid.pusher, c->np};
-    a.bbar_ready = 1;
     BbarPtrs<double> bg{{bb[0], bb[1], bb[2]}};
     {
       TimedScope ts(c, 1, 1);
@@ -813,15 +853,20 @@ pic_status window_after_step(pic_ctx* c) {
 // buffer), captured on first use; nullptr if capture is not possible.
 cudaGraphExec_t step_pair_graph(pic_ctx* c) {
   if (c->graphs_off) return nullptr;
+  // whether the pair's steps look for particles that left their windows
+  const bool strag = c->np > 0 && c->steps_since_sort + 1 > c->straggle_after;
   for (auto& g : c->sgraph)
-    if (g.exec && g.epoch == c->epoch && g.cur == c->cur && g.pcur == c->pcur) return g.exec;
+    if (g.exec && g.epoch == c->epoch && g.cur == c->cur && g.pcur == c->pcur && g.strag == strag)
+      return g.exec;
   // capture: run the two steps' launches into a graph, then restore the host
   // bookkeeping they advanced (it is advanced again at each replay)
   const int cur = c->cur, pcur = c->pcur, sss = c->steps_since_sort;
   const int64_t done = c->steps_done;
+  if (c->np == 0 && !c->j_zero) return nullptr;   // a plain step clears the current first
   cudaGraph_t gr = nullptr;
   cudaGraphExec_t ex = nullptr;
   bool ok = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+  c->strag_always = strag;
   if (ok) {
     pic_status s1 = step_once(c);
     pic_status s2 = s1 == PIC_OK ? step_once(c) : s1;
@@ -830,6 +875,7 @@ cudaGraphExec_t step_pair_graph(pic_ctx* c) {
   }
   if (gr) cudaGraphDestroy(gr);
   cudaGetLastError();  // a failed capture leaves no sticky error
+  c->strag_always = false;
   c->cur = cur;
   c->pcur = pcur;
   c->steps_since_sort = sss;
@@ -841,13 +887,13 @@ cudaGraphExec_t step_pair_graph(pic_ctx* c) {
   }
   // keep it in a free slot, or in place of one from an older epoch
   int slot = 0;
-  for (int k = 0; k < 4; ++k)
+  for (int k = 0; k < 8; ++k)
     if (!c->sgraph[k].exec || c->sgraph[k].epoch != c->epoch) {
       slot = k;
       break;
     }
   if (c->sgraph[slot].exec) cudaGraphExecDestroy(c->sgraph[slot].exec);
-  c->sgraph[slot] = pic_ctx::StepGraph{ex, cur, pcur, c->epoch};
+  c->sgraph[slot] = pic_ctx::StepGraph{ex, cur, pcur, strag, c->epoch};
   return ex;
 }
 
@@ -869,7 +915,11 @@ pic_status pic_step(pic_ctx* c, int64_t nsteps) {
     if (!c->timing && room >= 2) {
       cudaGraphExec_t ex = step_pair_graph(c);
       if (ex) {
-        const int64_t pairs = room / 2;
+        // as many pairs as keep the graph's kind (the last ones before a re-binning may
+        // have to look for particles that left their windows)
+        int64_t pairs = room / 2;
+        if (c->np > 0 && c->steps_since_sort < c->straggle_after)
+          pairs = std::min<int64_t>(pairs, (c->straggle_after - c->steps_since_sort + 1) / 2);
         for (int64_t k = 0; k < pairs; ++k) CK(c, cudaGraphLaunch(ex, c->stream));
         c->steps_since_sort += (int)(2 * pairs);
         c->steps_done += 2 * pairs;
@@ -1028,7 +1078,10 @@ pic_status pic_get_info(pic_ctx* c, pic_info* info) {
   info->correction_active = c->corr ? 1 : 0;
   info->cfl_lhs = c->cfl_lhs;
   info->cfl_sufficient_dt = c->cfl_suff;
-  info->kernels_per_step = 1 + (c->np > 0 ? (c->grid.ndim == 3 ? 3 : 2) : 0) + (c->corr ? 1 : 0);
+  const bool fused = c->grid.precision == PIC_FP64          ? field_step_fused<double>(c)
+                     : c->grid.precision == PIC_COMPENSATED ? field_step_fused<dfl>(c)
+                                                            : field_step_fused<float>(c);
+  info->kernels_per_step = c->np > 0 ? 3 + (c->corr ? 1 : 0) : (fused ? 1 : 2);
   return PIC_OK;
 }
 
@@ -1090,6 +1143,7 @@ pic_status pic_set_field_tile(pic_ctx* c, int t1, int t2, int t3, int threads, i
   c->ftile.t[2] = t3;
   c->ftile.threads = threads;
   c->ftile.staging = staging;
+  c->ftile_set = true;
   ++c->epoch;
   return PIC_OK;
 }
@@ -1118,6 +1172,7 @@ pic_status pic_set_field_strip(pic_ctx* c, int width, int rows, int warps, int s
   c->ftile.rows = rows;
   c->ftile.warps = warps;
   c->ftile.stages = stages;
+  c->ftile_set = true;
   ++c->epoch;
   return PIC_OK;
 }

@@ -20,7 +20,7 @@ struct FieldPtrs {
   T* j[3];
 };
 
-// time-centred B^n arrays (3D: formed once per step before the particle tiles)
+// time-centred B^n arrays (formed once per step before the particles)
 template <typename T>
 struct BbarPtrs {
   T* b[3];
@@ -92,6 +92,18 @@ cudaError_t launch_field_step(const FieldPtrs<T>& f, const FieldPtrs<T>& out, co
                               const StencilArgs<T>& s, const FieldTile& tile, unsigned* err,
                               cudaStream_t st);
 
+// The field step as two passes (field_halves.cu): Faraday of f into out.b -- with
+// bg (nullable) also the time-centred B into bg, zeros into f.j and into
+// *strag_count -- and Ampere of f.e and out.b into out.e with the current f.j (null
+// pointers: none).
+template <typename T>
+cudaError_t launch_faraday(const FieldPtrs<T>& f, const FieldPtrs<T>& out, const BbarPtrs<T>* bg,
+                           const GridArgs& g, const StencilArgs<T>& s,
+                           unsigned long long* strag_count, cudaStream_t st);
+template <typename T>
+cudaError_t launch_ampere(const FieldPtrs<T>& f, const FieldPtrs<T>& out, const GridArgs& g,
+                          const StencilArgs<T>& s, cudaStream_t st);
+
 template <typename T>
 cudaError_t launch_bbar(const FieldPtrs<T>& f, const GridArgs& g, const StencilArgs<T>& s,
                         double* out, int comp, cudaStream_t st);
@@ -142,9 +154,6 @@ struct PartArgs {
   double qm;
   int pusher;
   int64_t np;
-  // 1: the caller has formed the time-centred B in the BbarPtrs arrays (the
-  // spectral field path); the particle kernels read it there in 2D and 3D
-  int bbar_ready = 0;
 };
 
 struct BinBufs {

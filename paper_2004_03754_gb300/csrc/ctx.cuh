@@ -44,6 +44,8 @@ struct pic_ctx {
   int taps_lo = 0, taps_n = 0;
   int corr_path = 0;  // 0 automatic, 1 rows in place, 2 segments, 3 global
   FieldTile ftile{};
+  bool ftile_set = false;  // chosen by the caller: the fused field kernels always run
+  bool j_zero = true;      // the current arrays hold zeros (no deposit since they were cleared)
   // particles
   int64_t np = 0, cap = 0;
   double qm = -1.0;
@@ -53,6 +55,8 @@ struct pic_ctx {
   BinBufs bins{};
   int64_t bins_ntiles = 0;
   int sort_interval = 1;
+  bool strag_always = false;   // while a graph of steps past that point is captured
+  int straggle_after = 0;  // steps since a re-binning for which no particle can leave its window
   bool gain = false;  // energy-gain integrals per particle (Sec. 4.2) kept
   // moving window along x1 (Sec. 4.1): off while mw_start < 0; otherwise the
   // window moves at c from step mw_start of its own count on (mw_steps), and
@@ -72,13 +76,14 @@ struct pic_ctx {
   std::vector<cudaEvent_t> evpool;
   int64_t t_launches = 0, t_steps = 0;
   // CUDA graphs of two consecutive steps without re-binning, one per (field
-  // parity, particle buffer); dropped when the epoch changes (buffers or shapes)
+  // parity, particle buffer, straggler pass or not); dropped when the epoch changes (buffers or shapes)
   struct StepGraph {
     cudaGraphExec_t exec = nullptr;
     int cur = -1, pcur = -1;
+    bool strag = false;
     int64_t epoch = -1;
   };
-  StepGraph sgraph[4];
+  StepGraph sgraph[8];
   int64_t epoch = 0;
   bool graphs_off = false;  // set when a capture failed: plain launches from then on
 };
