@@ -54,6 +54,7 @@ struct BatchArgs {
   const int2* items;  // [0, nfield): (run, chunk*nstrips + strip); then (run, particle chunk);
                       // the last ncorr: (run, row) of the x1 current correction
   int nitems, nfield, ncorr;
+  int pchunk;         // particles per particle item: 1 (a warp each) or 32 (a lane each)
   const T* taps;      // correction taps of all row lengths (RunInfo::toff)
   unsigned* ctr;      // two per-step counters of taken field items (alternating steps)
   StripShape sh;
@@ -107,6 +108,16 @@ __device__ bool grid_wait(const BatchArgs<T>& A, unsigned& epoch) {
   return ok != 0;
 }
 
+// an accumulator at grid nodes offset from the caller's
+template <typename T>
+struct OffsetAcc {
+  GlobAcc<T> a;
+  int o1, o2;
+  __device__ __forceinline__ void add(int l1, int l2, int l3, typename DepositOf<T>::type v) const {
+    a.add(l1 + o1, l2 + o2, l3, v);
+  }
+};
+
 template <typename T>
 __device__ __forceinline__ T* pool_ptr(const BatchArgs<T>& A, int slot, int64_t off) {
   return A.pool + (int64_t)slot * A.total + off;
@@ -117,6 +128,90 @@ __device__ __forceinline__ T* pool_ptr(const BatchArgs<T>& A, int slot, int64_t 
 template <typename T>
 __device__ __forceinline__ T* run_ptr(const BatchArgs<T>& A, int slot, const RunInfo& R) {
   return pool_ptr(A, slot, R.off) + A.gh;
+}
+
+// One particle per warp.  A lone thread forming the time-centred B on the fly chains
+// some 600 loads of L2 latency, each behind index arithmetic, before a push: with 16
+// electrons per run that chain bounded the step (156 us for 16 runs).  Here the warp
+// evaluates the particle's 4x4 nodes of all six components at once -- a lane one node
+// of B2 or B3, whose x1 stencil it sums, and two of the others -- into its shared
+// memory, without wraps along x1 where the run's ghost columns hold the reach; lane 0
+// then advances the particle from there.  Every value takes the operations of
+// BbarView in their order.
+template <typename T>
+__device__ void particle_warp(const BatchArgs<T>& A, const StencilArgs<T>& s, const RunInfo& R,
+                              int64_t q, int par, int lane, T* buf) {
+  const int n1 = R.n1, n2 = R.n2, ld = R.ld;
+  int li[2];
+  T fr[2];
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    double frac;
+    li[d] = floor_split(A.parts.x[d][q] * A.gbase.inv_dx[d], frac);
+    fr[d] = to_prec<T>(frac);
+  }
+  const bool ghosted = n1 >= A.gh;
+  const T* E[3];
+  const T* B[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    E[c] = run_ptr(A, par * 6 + c, R);
+    B[c] = run_ptr(A, par * 6 + 3 + c, R);
+  }
+  auto row = [&](const T* a, int l2) { return a + (int64_t)wrap_index(l2, n2) * ld; };
+  auto val = [&](const T* r, int l1) { return gload<true>(r + (ghosted ? l1 : wrap_index(l1, n1))); };
+  {
+    // lanes 0-15: B2, 16-31: B3, at node (i, j) of the 4x4 window from cell - 1
+    const int i = li[0] - 1 + (lane & 3), j = li[1] - 1 + ((lane >> 2) & 3);
+    const bool b3 = lane >= 16;
+    const T* re = row(b3 ? E[1] : E[2], j);
+    T acc = 0;
+#pragma unroll 4
+    for (int m = 1; m <= s.M; ++m) acc += s.kE[m - 1] * (val(re, i + m) - val(re, i - m + 1));
+    T c;
+    if (b3) {
+      const T* r1 = row(E[0], j + 1);
+      const T* r0 = row(E[0], j);
+      c = acc - s.y2 * (val(r1, i) - val(r0, i));
+    } else {
+      c = -acc;
+    }
+    buf[(b3 ? 5 : 4) * 16 + (lane & 15)] = val(row(b3 ? B[2] : B[1], j), i) - (T)0.5 * c;
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {   // lanes 0-15: E1, E3; 16-31: E2, B1
+    const int i = li[0] - 1 + (lane & 3), j = li[1] - 1 + ((lane >> 2) & 3);
+    const int comp = lane < 16 ? 2 * h : (h == 0 ? 1 : 3);
+    T v;
+    if (comp == 3) {
+      const T c = s.y2 * (val(row(E[2], j + 1), i) - val(row(E[2], j), i));
+      v = val(row(B[0], j), i) - (T)0.5 * c;
+    } else {
+      v = val(row(comp == 0 ? E[0] : (comp == 1 ? E[1] : E[2]), j), i);
+    }
+    buf[comp * 16 + (lane & 15)] = v;
+  }
+  __syncwarp();
+  if (lane == 0) {
+    GridArgs g = A.gbase;
+    g.n[0] = n1;
+    g.n[1] = n2;
+    g.len[0] = n1 * g.dx[0];
+    g.len[1] = n2 * g.dx[1];
+    g.ncell = (int64_t)n1 * n2;
+    SmemView<T> ve[3], vb[3];
+    OffsetAcc<T> acc[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      ve[c] = SmemView<T>{buf + c * 16, 4, 16, 0};
+      vb[c] = SmemView<T>{buf + (3 + c) * 16, 4, 16, 0};
+      acc[c] = OffsetAcc<T>{GlobAcc<T>{run_ptr(A, 12 + c, R), n1, n2, 1, ld}, li[0] - 1, li[1] - 1};
+    }
+    const int l1[3] = {1, 1, 0}, gc[3] = {li[0], li[1], 0};
+    const T f3[3] = {fr[0], fr[1], (T)0};
+    advance_particle<T, 2, -1, false, true>(ve, vb, acc, A.parts, q, l1, f3, gc, g, A.a, A.err);
+  }
+  __syncwarp();
 }
 
 // 32 particles of a run per warp (gather E^n and time-centred B^n from the
@@ -433,8 +528,13 @@ __global__ void __launch_bounds__(256, 1) batch_kernel(BatchArgs<T> A) {
           const int2 w = A.items[A.nfield + k];
           const RunInfo R = A.runs[w.x];
           if (step >= R.nsteps) continue;
-          particle_chunk<T>(A, &s_sten, R, w.y, (R.cur + (int)step) & 1, lane);
+          const int par = (R.cur + (int)step) & 1;
+          if (A.pchunk == 1) particle_warp<T>(A, s_sten, R, R.p0 + w.y, par, lane, wbase);
+          else particle_chunk<T>(A, &s_sten, R, w.y, par, lane);
         }
+        // the field phase refills this shared memory with bulk copies
+        fence_proxy_async();
+        __syncwarp();
       }
       if (phase == 1 && nphase == 3) {
         for (int k = gw; k < A.ncorr; k += tw) {
@@ -532,6 +632,7 @@ struct pic_batch {
   int sw = 224, rows = 16, stages = 2, warps = 2;  // field strips (see StripShape)
   int gh = 0;  // ghost columns on each side of a pool row
   int nfield = 0;
+  int pchunk = 32;
   int corr = 0;              // C^B != e_1: the x1 current correction runs with the deposit
   void* taps = nullptr;      // correction taps of every row length, field precision
   int corr_elems = 0;        // shared-memory elements a warp needs for one corrected row
@@ -611,10 +712,15 @@ pic_status build_items(pic_batch* b) {
     for (int t = 0; t < nf; ++t) items.push_back(make_int2(r, t));
   }
   b->nfield = (int)items.size();
+  // a warp per particle while they are few beside the persistent kernel's warps (152
+  // SMs x 8): 16 runs of 16 electrons 154 -> 69 us per step, 24 runs 175 -> 90.  The
+  // chunks of 32 lanes, once hidden behind the field work, cost less in all: 60 runs
+  // (960 electrons) 206 us against 212, 256 runs 765 against 821.
+  b->pchunk = b->np <= 512 ? 1 : 32;
   for (int r = 0; r < b->nruns; ++r) {
     const RunInfo& R = b->runs[r];
     const int64_t n = R.p1 - R.p0;
-    const int chunks = (int)((n + 31) / 32);
+    const int chunks = (int)((n + b->pchunk - 1) / b->pchunk);
     for (int c = 0; c < chunks; ++c) items.push_back(make_int2(r, c));
   }
   b->ncorr = 0;
@@ -672,6 +778,7 @@ pic_status launch_batch(pic_batch* b) {
   A.sh = strip_shape(b);
   A.gh = b->gh;
   A.nfield = b->nfield;
+  A.pchunk = b->pchunk;
   A.ncorr = b->ncorr;
   A.taps = (const T*)b->taps;
   A.ctr = b->ctr;
@@ -843,6 +950,19 @@ pic_status pic_batch_init(const pic_batch_desc* d, double dt, const pic_coeffs* 
   b->rows = b->tsize == 4 ? 16 : 32;
   b->stages = 2;
   b->warps = 2;
+  {
+    // fewer rows per item, down to 4, while there are less than two items per warp of
+    // the persistent kernel (152 SMs x 8).  us per step with 16, 8 and 4 rows: 4 runs
+    // 58.6, 33.7, 31.5; 16 runs 69.3, 63.0, 55.6; 24 runs 89.9, 90.1, 84.6; 60 runs
+    // (three items of 16 rows per warp) 211.6, 214.1, 218.7
+    auto items = [&]() {
+      int64_t n = 0;
+      for (const RunInfo& R : b->runs)
+        n += (int64_t)((R.n1 + b->sw - 1) / b->sw) * ((R.n2 + b->rows - 1) / b->rows);
+      return n;
+    };
+    while (b->rows > 4 && items() < 2 * 152 * 8) b->rows /= 2;
+  }
   auto init_fail = [&](pic_status s) {
     pic_batch_destroy(b);
     return s;
