@@ -86,6 +86,7 @@ struct AdjPart {
   double* lx;              // 2 x n  adjoint of x
   double* lE[3];           // adjoint of E^n (scatter target)
   double* SB[3];           // scatter of the time-centred B adjoint
+  double* mB[3];           // magnetic adjoint (the warp kernel's local form)
   int64_t n;
   double qm;
   int pusher;              // PIC_BORIS or PIC_ANALYTIC
@@ -122,10 +123,119 @@ __device__ Vec3 deposit_adjoint(const AdjPart& A, int64_t q, const GridArgs& g, 
          (A.jscale * gj * w) * d2;
 }
 
-// One reverse step of the test particles of a 2D run (PUSH: the pusher).
+// Reverse push and move of particle q: gathers the six components and their
+// x-gradients (App. A) from `nodes`, replaces the particle's adjoints lu, lx by those
+// one step earlier and returns the adjoint of the gathered fields.  ax: the axes of
+// the nodes' indices.
+template <int PUSH, class NODES>
+__device__ void reverse_particle(const AdjPart& A, int64_t q, const GridArgs& g, const AxisD* ax,
+                                 const NODES& nodes, double leb[6]) {
+  constexpr int half[6][2] = {{1, 0}, {0, 1}, {0, 0}, {0, 1}, {1, 0}, {1, 1}};
+  double eb[6], g1[6], g2[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const int b1 = half[c][0] ? ax[0].bh : ax[0].bn;
+    const int b2 = half[c][1] ? ax[1].bh : ax[1].bn;
+    const double* w1 = half[c][0] ? ax[0].wh : ax[0].wn;
+    const double* w2 = half[c][1] ? ax[1].wh : ax[1].wn;
+    const double* d1 = half[c][0] ? ax[0].dwh : ax[0].dwn;
+    const double* d2 = half[c][1] ? ax[1].dwh : ax[1].dwn;
+    double v = 0, a1 = 0, a2 = 0;
+    for (int j = 0; j < 3; ++j)
+      for (int i = 0; i < 3; ++i) {
+        const double F = nodes.at(c, b1 + i, b2 + j);
+        v += F * w1[i] * w2[j];
+        a1 += F * d1[i] * w2[j];
+        a2 += F * w1[i] * d2[j];
+      }
+    eb[c] = v;
+    g1[c] = a1 * g.inv_dx[0];
+    g2[c] = a2 * g.inv_dx[1];
+  }
+  const Vec3 lxn = v3(A.lx[q], A.lx[A.n + q], 0.0);
+  const Vec3 lu_in = v3(A.lu[q], A.lu[A.n + q], A.lu[2 * A.n + q]);
+  double ldx[2] = {0.0, 0.0};   // deposit's share of the x^n adjoint
+  Vec3 lum;
+  if constexpr (PUSH == PIC_ANALYTIC) {
+    // analytic push: its Jacobian by dual numbers through the smooth form
+    const double u0[3] = {A.u[q], A.u[A.n + q], A.u[2 * A.n + q]};
+    double uo[3], jac[3][9];
+    analytic_push_jacobian(A.qm, g.dt, eb, u0, uo, jac);
+    const Vec3 un = v3(uo[0], uo[1], uo[2]);
+    const double gn = sqrt(1.0 + dot(un, un));
+    const Vec3 lun = lu_in + (g.dt / gn) * (lxn - (dot(un, lxn) / (gn * gn)) * un) +
+                     deposit_adjoint(A, q, g, un, gn, ldx);
+    double lk[9];
+    for (int k = 0; k < 9; ++k) lk[k] = lun.x * jac[0][k] + lun.y * jac[1][k] + lun.z * jac[2][k];
+    lum = v3(lk[0], lk[1], lk[2]);
+    for (int c = 0; c < 6; ++c) leb[c] = lk[3 + c];
+  } else {
+  // forward Boris with intermediates
+  const double h = 0.5 * A.qm * g.dt;
+  const Vec3 E = v3(eb[0], eb[1], eb[2]), B = v3(eb[3], eb[4], eb[5]);
+  const Vec3 u = v3(A.u[q], A.u[A.n + q], A.u[2 * A.n + q]);
+  const Vec3 um = u + h * E;
+  const double ig = 1.0 / sqrt(1.0 + dot(um, um));
+  const double hig = h * ig;
+  const Vec3 t = hig * B;
+  const double tt = dot(t, t);
+  const double f = 2.0 / (1.0 + tt);
+  const Vec3 sv = f * t;
+  const Vec3 p = um + cross(um, t);
+  const Vec3 up = um + cross(p, sv);
+  const Vec3 un = up + h * E;
+  const double gn = sqrt(1.0 + dot(un, un));
+  // reverse
+  // x^{n+1} = x^n + dt un/gn:  d(un/gn)/dun = (I - un un^T/gn^2)/gn
+  const Vec3 lun = lu_in + (g.dt / gn) * (lxn - (dot(un, lxn) / (gn * gn)) * un) +
+                   deposit_adjoint(A, q, g, un, gn, ldx);
+  Vec3 lE = h * lun;
+  const Vec3 lup = lun;
+  lum = lup;
+  const Vec3 lp = cross(sv, lup);
+  const Vec3 ls = cross(lup, p);
+  const double lf = dot(ls, t);
+  Vec3 lt = f * ls;
+  const double ltt = lf * (-0.5 * f * f);
+  lt = lt + (2.0 * ltt) * t;
+  lum = lum + lp + cross(t, lp);
+  lt = lt + cross(lp, um);
+  const Vec3 lB = hig * lt;
+  const double lhig = dot(lt, B);
+  lum = lum - (h * lhig * ig * ig * ig) * um;
+  lE = lE + h * lum;
+  leb[0] = lE.x; leb[1] = lE.y; leb[2] = lE.z;
+  leb[3] = lB.x; leb[4] = lB.y; leb[5] = lB.z;
+  }
+  // position adjoint: identity from x^{n+1} = x^n + ..., plus the field gradient
+  double lx1 = lxn.x + ldx[0], lx2 = lxn.y + ldx[1];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    lx1 += leb[c] * g1[c];
+    lx2 += leb[c] * g2[c];
+  }
+  A.lu[q] = lum.x;
+  A.lu[A.n + q] = lum.y;
+  A.lu[2 * A.n + q] = lum.z;
+  A.lx[q] = lx1;
+  A.lx[A.n + q] = lx2;
+}
+
+// node values straight from global memory, the time-centred B formed on the fly
+struct AdjGlobal {
+  GlobView<double> ve[3];
+  BbarView<double, 2> vb[3];
+  __device__ __forceinline__ double at(int c, int i, int j) const {
+    return c < 3 ? ve[c].at(i, j, 0) : vb[c - 3].at(i, j, 0);
+  }
+};
+
+// One reverse step of the particles of a 2D run, a thread per particle (PUSH: the
+// pusher); the time-centred B's adjoint is left in A.SB.
 template <int PUSH>
 __global__ void adjoint_particle_kernel(AdjPart A, GridArgs g, StencilArgs<double> s) {
   const int n1 = g.n[0], n2 = g.n[1];
+  constexpr int half[6][2] = {{1, 0}, {0, 1}, {0, 0}, {0, 1}, {1, 0}, {1, 1}};
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < A.n;
        q += (int64_t)gridDim.x * blockDim.x) {
     AxisD ax[2];
@@ -134,103 +244,13 @@ __global__ void adjoint_particle_kernel(AdjPart A, GridArgs g, StencilArgs<doubl
       const double fl = floor(c);
       axis_d((int)fl, c - fl, ax[d]);
     }
-    GlobView<double> ve[3];
-    BbarView<double, 2> vb[3];
+    AdjGlobal nodes;
     for (int c = 0; c < 3; ++c) {
-      ve[c] = GlobView<double>{A.F[c], n1, n2, 1, n1};
-      vb[c] = BbarView<double, 2>{{A.F[0], A.F[1], A.F[2]}, A.F[3 + c], c, n1, n2, 1, &s, n1};
+      nodes.ve[c] = GlobView<double>{A.F[c], n1, n2, 1, n1};
+      nodes.vb[c] = BbarView<double, 2>{{A.F[0], A.F[1], A.F[2]}, A.F[3 + c], c, n1, n2, 1, &s, n1};
     }
-    // gather of the six components and their x-gradients (App. A)
-    constexpr int half[6][2] = {{1, 0}, {0, 1}, {0, 0}, {0, 1}, {1, 0}, {1, 1}};
-    double eb[6], g1[6], g2[6];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      const int b1 = half[c][0] ? ax[0].bh : ax[0].bn;
-      const int b2 = half[c][1] ? ax[1].bh : ax[1].bn;
-      const double* w1 = half[c][0] ? ax[0].wh : ax[0].wn;
-      const double* w2 = half[c][1] ? ax[1].wh : ax[1].wn;
-      const double* d1 = half[c][0] ? ax[0].dwh : ax[0].dwn;
-      const double* d2 = half[c][1] ? ax[1].dwh : ax[1].dwn;
-      double v = 0, a1 = 0, a2 = 0;
-      for (int j = 0; j < 3; ++j)
-        for (int i = 0; i < 3; ++i) {
-          const double F = c < 3 ? ve[c].at(b1 + i, b2 + j, 0) : vb[c - 3].at(b1 + i, b2 + j, 0);
-          v += F * w1[i] * w2[j];
-          a1 += F * d1[i] * w2[j];
-          a2 += F * w1[i] * d2[j];
-        }
-      eb[c] = v;
-      g1[c] = a1 * g.inv_dx[0];
-      g2[c] = a2 * g.inv_dx[1];
-    }
-    const Vec3 lxn = v3(A.lx[q], A.lx[A.n + q], 0.0);
-    const Vec3 lu_in = v3(A.lu[q], A.lu[A.n + q], A.lu[2 * A.n + q]);
     double leb[6];
-    double ldx[2] = {0.0, 0.0};   // deposit's share of the x^n adjoint
-    Vec3 lum;
-    if constexpr (PUSH == PIC_ANALYTIC) {
-      // analytic push: its Jacobian by dual numbers through the smooth form
-      const double u0[3] = {A.u[q], A.u[A.n + q], A.u[2 * A.n + q]};
-      double uo[3], jac[3][9];
-      analytic_push_jacobian(A.qm, g.dt, eb, u0, uo, jac);
-      const Vec3 un = v3(uo[0], uo[1], uo[2]);
-      const double gn = sqrt(1.0 + dot(un, un));
-      const Vec3 lun = lu_in + (g.dt / gn) * (lxn - (dot(un, lxn) / (gn * gn)) * un) +
-                       deposit_adjoint(A, q, g, un, gn, ldx);
-      double lk[9];
-      for (int k = 0; k < 9; ++k) lk[k] = lun.x * jac[0][k] + lun.y * jac[1][k] + lun.z * jac[2][k];
-      lum = v3(lk[0], lk[1], lk[2]);
-      for (int c = 0; c < 6; ++c) leb[c] = lk[3 + c];
-    } else {
-    // forward Boris with intermediates
-    const double h = 0.5 * A.qm * g.dt;
-    const Vec3 E = v3(eb[0], eb[1], eb[2]), B = v3(eb[3], eb[4], eb[5]);
-    const Vec3 u = v3(A.u[q], A.u[A.n + q], A.u[2 * A.n + q]);
-    const Vec3 um = u + h * E;
-    const double ig = 1.0 / sqrt(1.0 + dot(um, um));
-    const double hig = h * ig;
-    const Vec3 t = hig * B;
-    const double tt = dot(t, t);
-    const double f = 2.0 / (1.0 + tt);
-    const Vec3 sv = f * t;
-    const Vec3 p = um + cross(um, t);
-    const Vec3 up = um + cross(p, sv);
-    const Vec3 un = up + h * E;
-    const double gn = sqrt(1.0 + dot(un, un));
-    // reverse
-    // x^{n+1} = x^n + dt un/gn:  d(un/gn)/dun = (I - un un^T/gn^2)/gn
-    const Vec3 lun = lu_in + (g.dt / gn) * (lxn - (dot(un, lxn) / (gn * gn)) * un) +
-                     deposit_adjoint(A, q, g, un, gn, ldx);
-    Vec3 lE = h * lun;
-    const Vec3 lup = lun;
-    lum = lup;
-    const Vec3 lp = cross(sv, lup);
-    const Vec3 ls = cross(lup, p);
-    const double lf = dot(ls, t);
-    Vec3 lt = f * ls;
-    const double ltt = lf * (-0.5 * f * f);
-    lt = lt + (2.0 * ltt) * t;
-    lum = lum + lp + cross(t, lp);
-    lt = lt + cross(lp, um);
-    const Vec3 lB = hig * lt;
-    const double lhig = dot(lt, B);
-    lum = lum - (h * lhig * ig * ig * ig) * um;
-    lE = lE + h * lum;
-    leb[0] = lE.x; leb[1] = lE.y; leb[2] = lE.z;
-    leb[3] = lB.x; leb[4] = lB.y; leb[5] = lB.z;
-    }
-    // position adjoint: identity from x^{n+1} = x^n + ..., plus the field gradient
-    double lx1 = lxn.x + ldx[0], lx2 = lxn.y + ldx[1];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      lx1 += leb[c] * g1[c];
-      lx2 += leb[c] * g2[c];
-    }
-    A.lu[q] = lum.x;
-    A.lu[A.n + q] = lum.y;
-    A.lu[2 * A.n + q] = lum.z;
-    A.lx[q] = lx1;
-    A.lx[A.n + q] = lx2;
+    reverse_particle<PUSH>(A, q, g, ax, nodes, leb);
     // transpose of the gather: scatter with the same weights
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
@@ -247,27 +267,116 @@ __global__ void adjoint_particle_kernel(AdjPart A, GridArgs g, StencilArgs<doubl
   }
 }
 
-// E += alpha * K_B[c] S  (Ampere-form curl, d^B stencil with coefficients pre-scaled
-// in s.kE, i.e. dt C^E / dx1; alpha carries the remaining factor)
-__global__ void curl_b_axpy_kernel(double* E0, double* E1, double* E2, const double* S0,
-                                   const double* S1, const double* S2, GridArgs g,
-                                   StencilArgs<double> s, double alpha) {
+// The same reverse step with a warp per particle.  A lone thread chains some 600 loads
+// for the time-centred B's stencils and the scatters one after another; here the lanes
+// evaluate the particle's 4x4 nodes of the six components into shared memory (a lane
+// one node of B2 or B3, whose x1 stencil it sums, and two of the others), lane 0 runs
+// the reverse push from there and the lanes scatter.  LOCAL: the time-centred B's
+// adjoint S (27 nodes) goes straight through its transposed curl into lE, -(1/2)
+// K_B[C^E] S, and into the magnetic adjoint, m_B -= S, by atomics around the particle
+// (some 260) instead of by passes over the grid.
+struct AdjNodes {
+  const double* v;   // [6][16]: component, node (i, j) of the 4x4 window
+  __device__ __forceinline__ double at(int c, int i, int j) const { return v[c * 16 + j * 4 + i]; }
+};
+
+template <int PUSH, bool LOCAL>
+__global__ void __launch_bounds__(128) adjoint_particle_warp_kernel(AdjPart A, GridArgs g,
+                                                                    StencilArgs<double> s) {
+  __shared__ double sm[4][112];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int n1 = g.n[0], n2 = g.n[1];
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.ncell;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(q % n1), j = (int)(q / n1);
-    auto at = [&](const double* a, int di, int dj) {
-      return a[(int64_t)wrap_index(j + dj, n2) * n1 + wrap_index(i + di, n1)];
-    };
-    double dS2 = 0, dS3 = 0;
-    for (int m = 1; m <= s.M; ++m) {
-      dS3 += s.kE[m - 1] * (at(S2, m - 1, 0) - at(S2, -m, 0));
-      dS2 += s.kE[m - 1] * (at(S1, m - 1, 0) - at(S1, -m, 0));
+  double* buf = sm[wib];
+  double* out = buf + 96;   // leb[6]
+  for (int64_t q = blockIdx.x * 4ll + wib; q < A.n; q += gridDim.x * 4ll) {
+    AxisD ax[2];
+    int li[2];
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      const double c = A.x[d * A.n + q] * g.inv_dx[d];
+      const double fl = floor(c);
+      li[d] = (int)fl;
+      axis_d(1, c - fl, ax[d]);   // window-local: the cell is node 1
     }
-    const double y2 = s.y2;
-    E0[q] += alpha * (y2 * (at(S2, 0, 0) - at(S2, 0, -1)));
-    E1[q] += alpha * (-dS3);
-    E2[q] += alpha * (dS2 - y2 * (at(S0, 0, 0) - at(S0, 0, -1)));
+    auto at = [&](const double* a, int i, int j) {
+      return a[(int64_t)wrap_index(j, n2) * n1 + wrap_index(i, n1)];
+    };
+    const int i = li[0] - 1 + (lane & 3), j = li[1] - 1 + ((lane >> 2) & 3);
+    {
+      const bool b3 = lane >= 16;
+      const double* a = (b3 ? A.F[1] : A.F[2]) + (int64_t)wrap_index(j, n2) * n1;
+      double acc = 0.0;
+      int ip = wrap_index(i + 1, n1), im = wrap_index(i, n1);
+#pragma unroll 4
+      for (int m = 0; m < s.M; ++m) {
+        acc += s.kE[m] * (a[ip] - a[im]);
+        if (++ip == n1) ip = 0;
+        if (--im < 0) im = n1 - 1;
+      }
+      const double c = b3 ? acc - s.y2 * (at(A.F[0], i, j + 1) - at(A.F[0], i, j)) : -acc;
+      buf[(b3 ? 5 : 4) * 16 + (lane & 15)] = at(b3 ? A.F[5] : A.F[4], i, j) - 0.5 * c;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int comp = lane < 16 ? 2 * h : (h == 0 ? 1 : 3);
+      double v = at(comp == 0 ? A.F[0] : (comp == 1 ? A.F[1] : (comp == 2 ? A.F[2] : A.F[3])), i, j);
+      if (comp == 3) v -= 0.5 * (s.y2 * (at(A.F[2], i, j + 1) - at(A.F[2], i, j)));
+      buf[comp * 16 + (lane & 15)] = v;
+    }
+    __syncwarp();
+    if (lane == 0) {
+      const AdjNodes nodes{buf};
+      double leb[6];
+      reverse_particle<PUSH>(A, q, g, ax, nodes, leb);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) out[c] = leb[c];
+    }
+    __syncwarp();
+    auto add = [&](double* a, int ii, int jj, double v) {
+      atomicAdd(&a[(int64_t)wrap_index(jj, n2) * n1 + wrap_index(ii, n1)], v);
+    };
+    const int o1 = li[0] - 1, o2 = li[1] - 1;   // grid node of window node 0
+    auto wt = [&](int c, int a, int b) {        // weight of node (a, b) of component c's 3x3
+      constexpr int half[6][2] = {{1, 0}, {0, 1}, {0, 0}, {0, 1}, {1, 0}, {1, 1}};
+      return (half[c][0] ? ax[0].wh[a] : ax[0].wn[a]) * (half[c][1] ? ax[1].wh[b] : ax[1].wn[b]);
+    };
+    auto b1 = [&](int c) { return (c == 0 || c == 4 || c == 5) ? ax[0].bh : ax[0].bn; };
+    auto b2 = [&](int c) { return (c == 1 || c == 3 || c == 5) ? ax[1].bh : ax[1].bn; };
+    for (int k = lane; k < 54; k += 32) {
+      const int c = k / 9, r = k - 9 * c, b = r / 3, a = r - 3 * b;
+      const double v = out[c] * wt(c, a, b);
+      const int ii = o1 + b1(c) + a, jj = o2 + b2(c) + b;
+      if (c < 3) add(A.lE[c], ii, jj, v);
+      else if (LOCAL) add(A.mB[c - 3], ii, jj, -v);
+      else add(A.SB[c - 3], ii, jj, v);
+    }
+    if constexpr (LOCAL) {
+      // E1 += -(y2/2) (S3_j - S3_{j-1}), E3 += (y2/2) (S1_j - S1_{j-1}): rows of the
+      // 3x3 and the one above
+      if (lane < 24) {
+        const int c = lane < 12 ? 5 : 3, r = lane % 12, b = r / 3, a = r - 3 * b;
+        const double sj = b < 3 ? wt(c, a, b) : 0.0, sm1 = b > 0 ? wt(c, a, b - 1) : 0.0;
+        const double v = 0.5 * s.y2 * out[c] * (sj - sm1);
+        add(A.lE[c == 5 ? 0 : 2], o1 + b1(c) + a, o2 + b2(c) + b, c == 5 ? -v : v);
+      }
+      // E2 += (1/2) d_B-form S3, E3 += -(1/2) d_B-form S2 along x1: node i reaches the
+      // outputs i - M + 1 .. i (taps +k) and i + 1 .. i + M (taps -k)
+      const int cols = 2 * s.M + 2;
+      for (int k = lane; k < 6 * cols; k += 32) {
+        const int cr = k / cols, col = k - cr * cols - (s.M - 1);   // column relative to the 3x3
+        const int c = cr < 3 ? 5 : 4, b = cr < 3 ? cr : cr - 3;
+        double acc = 0.0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int m = a - col;   // node minus output
+          if (m >= 0 && m < s.M) acc += s.kE[m] * wt(c, a, b);
+          else if (m < 0 && -m <= s.M) acc -= s.kE[-m - 1] * wt(c, a, b);
+        }
+        const double v = 0.5 * out[c] * acc;
+        add(A.lE[c == 5 ? 1 : 2], o1 + b1(c) + col, o2 + b2(c) + b, c == 5 ? v : -v);
+      }
+    }
+    __syncwarp();
   }
 }
 
@@ -412,6 +521,47 @@ pic_status load_fields(pic_ctx* c, double* const* src) {
   return PIC_OK;
 }
 
+// One forward step between field states kept by the adjoint: no copies on the plain
+// stencil path; the spectral path and the moving window step the context's own fields.
+pic_status forward_step(pic_ctx* c, double* const* fin, double* const* fout) {
+  if (!c->spec && c->mw_start < 0) return step_between(c, fin, fout);
+  PCK(load_fields(c, fin));
+  PCK(pic_step(c, 1));
+  return save_fields(c, fout);
+}
+
+// One reverse step of the field adjoint (lE, mB) -> (lE', mB'): the forward passes with
+// the stencils of sw and no current.
+pic_status reverse_fields(pic_ctx* c, double* const* lE, double* const* mB, double* const* lEo,
+                          double* const* mBo, const StencilArgs<double>& sw) {
+  FieldPtrs<double> f{}, o{};
+  for (int m = 0; m < 3; ++m) {
+    f.e[m] = lE[m];
+    f.b[m] = mB[m];
+    o.e[m] = lEo[m];
+    o.b[m] = mBo[m];
+  }
+  ACK(c, launch_faraday<double>(f, o, nullptr, c->g, sw, nullptr, c->stream));
+  ACK(c, launch_ampere<double>(f, o, c->g, sw, c->stream));
+  return PIC_OK;
+}
+
+// E += alpha K_B[c] S, in place (Ampere-form curl, d^B stencil with the coefficients of
+// s.kE, i.e. dt C^E / dx1; alpha carries the remaining factor)
+pic_status curl_b_axpy(pic_ctx* c, double* const* E, double* const* S, double alpha) {
+  StencilArgs<double> a = c->sd;
+  for (int j = 0; j < PIC_MAX_M; ++j) a.kB[j] = alpha * c->sd.kE[j];
+  a.y2 = alpha * c->sd.y2;
+  a.y3 = alpha * c->sd.y3;
+  FieldPtrs<double> f{}, o{};
+  for (int m = 0; m < 3; ++m) {
+    f.e[m] = o.e[m] = E[m];
+    o.b[m] = S[m];
+  }
+  ACK(c, launch_ampere<double>(f, o, c->g, a, c->stream));
+  return PIC_OK;
+}
+
 StencilArgs<double> swapped(const pic_ctx* c) {
   StencilArgs<double> s = c->sd;
   for (int j = 0; j < PIC_MAX_M; ++j) std::swap(s.kE[j], s.kB[j]);
@@ -454,13 +604,16 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
       ACK(c, P.get(&muB[s][k], nc));
     }
   for (int k = 0; k < 3; ++k) ACK(c, P.get(&SB[k], nc));
+  double* finF[6] = {nullptr};   // final fields where the context's own are stepped again
+  if (c->spec || c->mw_start >= 0)
+    for (int k = 0; k < 6; ++k) ACK(c, P.get(&finF[k], nc));
   std::vector<double*> ckf((size_t)nseg * 6), ckx(nseg), cku(nseg);
-  for (int s = 0; s < nseg; ++s) {
+  for (int s = 0; s + 1 < nseg; ++s) {
     for (int k = 0; k < 6; ++k) ACK(c, P.get(&ckf[(size_t)s * 6 + k], nc));
     ACK(c, P.get(&ckx[s], 2 * n));
     ACK(c, P.get(&cku[s], 3 * n));
   }
-  double *segF, *segx, *segu, *lu, *lx, *wz, *acc, *uend, *xend, *finF[6];
+  double *segF, *segx, *segu, *lu, *lx, *wz, *acc, *uend, *xend;
   ACK(c, P.get(&segF, (size_t)seg * 6 * nc));
   ACK(c, P.get(&segx, (size_t)seg * 2 * n));
   ACK(c, P.get(&segu, (size_t)seg * 3 * n));
@@ -470,7 +623,6 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
   ACK(c, P.get(&acc, 4));
   ACK(c, P.get(&uend, 3 * n));
   ACK(c, P.get(&xend, 2 * n));
-  for (int k = 0; k < 6; ++k) ACK(c, P.get(&finF[k], nc));
   cudaStream_t st = c->stream;
   ACK(c, cudaMemsetAsync(wz, 0, sizeof(double) * n, st));
   // weights on the device (the segment recomputations load from device arrays)
@@ -507,14 +659,52 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
     PCK(pic_load_particles(c, n, x, u, w ? w : w0.data(), -1.0, 0));
   }
   const double qm = c->qm;
-  // forward with checkpoints
+  auto state = [&](int64_t k, double** f) {   // field state k of the segment in memory
+    for (int m = 0; m < 6; ++m) f[m] = segF + ((size_t)k * 6 + m) * nc;
+  };
+  // the steps of one segment from its field state 0, the field states 0 .. steps-1 and
+  // the particles of every step kept; the last step goes into `last` (null: not taken)
+  auto segment = [&](int64_t steps, double* const* last) -> pic_status {
+    for (int64_t k = 0; k < steps; ++k) {
+      PCK(pic_read_particles(c, segx + (size_t)k * 2 * n, segu + (size_t)k * 3 * n, nullptr, 1));
+      double *fi[6], *fo[6];
+      state(k, fi);
+      if (k + 1 < steps) {
+        state(k + 1, fo);
+        PCK(forward_step(c, fi, fo));
+      } else if (last) {
+        PCK(forward_step(c, fi, last));
+      }
+    }
+    return PIC_OK;
+  };
+  // forward with checkpoints; the last segment's states stay in memory
   for (int s = 0; s < nseg; ++s) {
-    PCK(save_fields(c, &ckf[(size_t)s * 6]));
-    PCK(pic_read_particles(c, ckx[s], cku[s], nullptr, 1));
-    PCK(pic_step(c, std::min<int64_t>(ckp, nsteps - (int64_t)s * ckp)));
+    const int64_t steps = std::min<int64_t>(ckp, nsteps - (int64_t)s * ckp);
+    if (s + 1 < nseg) {
+      PCK(save_fields(c, &ckf[(size_t)s * 6]));
+      PCK(pic_read_particles(c, ckx[s], cku[s], nullptr, 1));
+      PCK(pic_step(c, steps));
+    } else {
+      double *f0[6], *fin[6];
+      state(0, f0);
+      PCK(save_fields(c, f0));
+      for (int m = 0; m < 3; ++m) {
+        fin[m] = (double*)c->fe[1 - c->cur][m];
+        fin[3 + m] = (double*)c->fb[1 - c->cur][m];
+      }
+      const bool own = !c->spec && c->mw_start < 0;   // the context's fields don't move meanwhile
+      PCK(segment(steps, own ? fin : finF));
+      if (own) {
+        c->cur = 1 - c->cur;
+        c->steps_done += steps;
+      }
+    }
   }
   PCK(pic_read_particles(c, xend, uend, nullptr, 1));
-  PCK(save_fields(c, finF));
+  if (c->spec || c->mw_start >= 0) PCK(load_fields(c, finF));
+  const bool warp = n <= 8192;             // a warp per particle
+  const bool local = warp && n <= nc / 256;   // its curl by atomics (260 per particle), not by grid passes
   ACK(c, cudaMemsetAsync(acc, 0, sizeof(double) * 4, st));
   energy_sum_kernel<<<nblk(n), 256, 0, st>>>(uend, n, acc);
   energy_seed_kernel<<<nblk(n), 256, 0, st>>>(uend, lu, lx, n);
@@ -528,31 +718,18 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
   int a = 0;  // adjoint buffer parity
   for (int s = nseg - 1; s >= 0; --s) {
     const int64_t n0 = (int64_t)s * ckp, n1 = std::min<int64_t>(nsteps, n0 + ckp);
-    PCK(load_fields(c, &ckf[(size_t)s * 6]));
-    PCK(pic_load_particles(c, n, ckx[s], cku[s], wdev, qm, 1));
-    for (int64_t k = n0; k < n1; ++k) {
-      double* dst[6];
-      for (int m = 0; m < 6; ++m) dst[m] = segF + ((size_t)(k - n0) * 6 + m) * nc;
-      PCK(save_fields(c, dst));
-      PCK(pic_read_particles(c, segx + (size_t)(k - n0) * 2 * n, segu + (size_t)(k - n0) * 3 * n,
-                             nullptr, 1));
-      PCK(pic_step(c, 1));
+    if (s + 1 < nseg) {
+      double* f0[6];
+      state(0, f0);
+      for (int m = 0; m < 6; ++m)
+        ACK(c, cudaMemcpyAsync(f0[m], ckf[(size_t)s * 6 + m], sizeof(double) * nc,
+                               cudaMemcpyDeviceToDevice, st));
+      PCK(pic_load_particles(c, n, ckx[s], cku[s], wdev, qm, 1));
+      PCK(segment(n1 - n0, nullptr));
     }
-    // the transposed field step below runs with no current
-    for (int m = 0; m < 3; ++m)
-      ACK(c, cudaMemsetAsync(c->fj[m], 0, sizeof(double) * nc, st));
     for (int64_t k = n1 - 1; k >= n0; --k) {
       // fields: l^k = A^T l^{k+1}
-      FieldPtrs<double> fi, fo;
-      for (int m = 0; m < 3; ++m) {
-        fi.e[m] = lamE[a][m];
-        fi.b[m] = muB[a][m];
-        fi.j[m] = (double*)c->fj[m];  // zero (cleared above)
-        fo.e[m] = lamE[1 - a][m];
-        fo.b[m] = muB[1 - a][m];
-        fo.j[m] = (double*)c->fj[m];
-      }
-      ACK(c, launch_field_step<double>(fi, fo, c->g, sw, c->ftile, c->bins.err, st));
+      PCK(reverse_fields(c, lamE[a], muB[a], lamE[1 - a], muB[1 - a], sw));
       a = 1 - a;
       // particles at step k
       AdjPart A;
@@ -579,15 +756,26 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
                                          c->taps_n, c->corr_path, st));
         A.lJ[0] = tmpJ1;
       }
-      if (A.pusher == PIC_ANALYTIC)
-        adjoint_particle_kernel<PIC_ANALYTIC><<<nblk(n), 128, 0, st>>>(A, c->g, c->sd);
-      else
-        adjoint_particle_kernel<PIC_BORIS><<<nblk(n), 128, 0, st>>>(A, c->g, c->sd);
-      // time-centred B: l_B += S, l_E += -(1/2) K_B[C^E] S  (m_B = -l_B)
-      curl_b_axpy_kernel<<<nblk(nc), 256, 0, st>>>(lamE[a][0], lamE[a][1], lamE[a][2], SB[0],
-                                                   SB[1], SB[2], c->g, c->sd, -0.5);
-      sub_clear_kernel<<<nblk(nc), 256, 0, st>>>(muB[a][0], muB[a][1], muB[a][2], SB[0], SB[1],
-                                                 SB[2], nc);
+      for (int m = 0; m < 3; ++m) A.mB[m] = muB[a][m];
+      const int nbw = (int)std::min<int64_t>((n + 3) / 4, 152 * 16);
+      const bool an = A.pusher == PIC_ANALYTIC;
+      if (local) {
+        if (an) adjoint_particle_warp_kernel<PIC_ANALYTIC, true><<<nbw, 128, 0, st>>>(A, c->g, c->sd);
+        else adjoint_particle_warp_kernel<PIC_BORIS, true><<<nbw, 128, 0, st>>>(A, c->g, c->sd);
+      } else {
+        if (warp && an)
+          adjoint_particle_warp_kernel<PIC_ANALYTIC, false><<<nbw, 128, 0, st>>>(A, c->g, c->sd);
+        else if (warp)
+          adjoint_particle_warp_kernel<PIC_BORIS, false><<<nbw, 128, 0, st>>>(A, c->g, c->sd);
+        else if (an)
+          adjoint_particle_kernel<PIC_ANALYTIC><<<nblk(n), 128, 0, st>>>(A, c->g, c->sd);
+        else
+          adjoint_particle_kernel<PIC_BORIS><<<nblk(n), 128, 0, st>>>(A, c->g, c->sd);
+        // time-centred B: l_B += S, l_E += -(1/2) K_B[C^E] S  (m_B = -l_B)
+        PCK(curl_b_axpy(c, lamE[a], SB, -0.5));
+        sub_clear_kernel<<<nblk(nc), 256, 0, st>>>(muB[a][0], muB[a][1], muB[a][2], SB[0], SB[1],
+                                                   SB[2], nc);
+      }
       ACK(c, cudaGetLastError());
     }
   }
@@ -613,7 +801,7 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
   *dJ_da0 = (h[1] - h[3]) / laser->a0;
   *dJ_dphase = h[2] - mB_F0p;
   // leave the state at the end of the forward run
-  PCK(load_fields(c, finF));
+  if (c->spec || c->mw_start >= 0) PCK(load_fields(c, finF));
   PCK(pic_load_particles(c, n, xend, uend, wdev, qm, 1));
   return pic_sync(c);
 }
@@ -707,16 +895,7 @@ extern "C" pic_status pic_adjoint_dispersion(pic_ctx* c, const double* e2_0, con
       // dJ/dC^B: <l_E^{k+1}, dE^{k+1}/dC^B> with B^{k+1/2}:  l_E3 DB B2 - l_E2 DB B3
       coeff_grad_kernel<PIC_MAX_M><<<nblk(nc), 256, 0, st>>>(
           lamE[a][2], lamE[a][1], Fk1 + 4 * nc, Fk1 + 5 * nc, c->g, M, 1, gB);
-      FieldPtrs<double> fi, fo;
-      for (int m = 0; m < 3; ++m) {
-        fi.e[m] = lamE[a][m];
-        fi.b[m] = muB[a][m];
-        fi.j[m] = (double*)c->fj[m];
-        fo.e[m] = lamE[1 - a][m];
-        fo.b[m] = muB[1 - a][m];
-        fo.j[m] = (double*)c->fj[m];
-      }
-      ACK(c, launch_field_step<double>(fi, fo, c->g, sw, c->ftile, c->bins.err, st));
+      PCK(reverse_fields(c, lamE[a], muB[a], lamE[1 - a], muB[1 - a], sw));
       a = 1 - a;
       // dJ/dC^E: <l_B'', dB'/dC^E> with l_B'' = -m_B^k:  l_B2 D E3 - l_B3 D E2
       //        = (-m_B3) ... written as  m_B3 D E2 - m_B2 D E3

@@ -261,13 +261,13 @@ bool field_step_fused(const pic_ctx* c) {
          c->g.ncell >= kFusedMinCells;
 }
 
+// One step from the fields f into o (f.j: the context's current).
 template <typename T>
-pic_status one_step(pic_ctx* c, const StencilArgs<T>& s) {
+pic_status step_fields(pic_ctx* c, const StencilArgs<T>& s, FieldPtrs<T> f, const FieldPtrs<T>& o) {
   if (c->steps_since_sort >= c->sort_interval) {
     pic_status st = rebin(c);
     if (st != PIC_OK) return st;
   }
-  FieldPtrs<T> f = fields<T>(c, c->cur), o = fields<T>(c, 1 - c->cur);
   BbarPtrs<T> bg{{(T*)c->bbar[0], (T*)c->bbar[1], (T*)c->bbar[2]}};
   const bool parts = c->np > 0;
   if (!parts && !c->j_zero)
@@ -310,8 +310,15 @@ pic_status one_step(pic_ctx* c, const StencilArgs<T>& s) {
     }
   }
   if (c->timing) c->t_steps++;
-  c->cur = 1 - c->cur;
   c->steps_since_sort++;
+  return PIC_OK;
+}
+
+template <typename T>
+pic_status one_step(pic_ctx* c, const StencilArgs<T>& s) {
+  pic_status st = step_fields<T>(c, s, fields<T>(c, c->cur), fields<T>(c, 1 - c->cur));
+  if (st != PIC_OK) return st;
+  c->cur = 1 - c->cur;
   c->steps_done++;
   return PIC_OK;
 }
@@ -351,6 +358,17 @@ __global__ void check_positions_kernel(PartPtrs p, GridArgs g, int64_t np, unsig
 }
 
 }  // namespace
+
+pic_status step_between(pic_ctx* c, double* const* fin, double* const* fout) {
+  FieldPtrs<double> f = fields<double>(c, c->cur), o = f;
+  for (int k = 0; k < 3; ++k) {
+    f.e[k] = fin[k];
+    f.b[k] = fin[3 + k];
+    o.e[k] = fout[k];
+    o.b[k] = fout[3 + k];
+  }
+  return step_fields<double>(c, c->sd, f, o);
+}
 
 // Checkpoint layout (pic_save_state / pic_load_state): a header, then E1 E2 E3
 // B1 B2 B3 (n1*n2*n3 values each, field precision, x1 fastest), then the

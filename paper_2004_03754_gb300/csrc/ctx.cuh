@@ -88,6 +88,10 @@ struct pic_ctx {
   bool graphs_off = false;  // set when a capture failed: plain launches from then on
 };
 
+// api.cu (FP64 contexts on the stencil path): one step from the fields fin (E1 E2 E3
+// B1 B2 B3) into fout, with the context's particles and current
+pic_status step_between(pic_ctx* c, double* const* fin, double* const* fout);
+
 // spectral.cu (FP64 contexts)
 pic_status spectral_setup(pic_ctx* c, int nbins, const double* kE1, const double* kB1,
                           double slope0);

@@ -81,10 +81,10 @@ inline void laser_profiles(int n, double dx, double dt, int M, const double* cE,
   } else {
     for (int m = 0; m < n; ++m) {
       double a = 0, b = 0;
-      for (int i = 0; i < n; ++i) {
-        const int64_t r = (int64_t)m * i % n;
+      for (int i = 0, r = 0; i < n; ++i) {   // r = m i mod n
         a += ep[i] * cs[r];
         b -= ep[i] * sn[r];
+        if ((r += m) >= n) r -= n;
       }
       fa[m] = a;
       fb[m] = b;
@@ -117,9 +117,9 @@ inline void laser_profiles(int n, double dx, double dt, int M, const double* cE,
   }
   for (int i = 0; i < n; ++i) {
     double s = 0;
-    for (int m = 0; m < n; ++m) {
-      const int64_t r = (int64_t)m * i % n;
+    for (int m = 0, r = 0; m < n; ++m) {   // r = m i mod n
       s += re[m] * cs[r] - im[m] * sn[r];
+      if ((r += i) >= n) r -= n;
     }
     bp[i] = s / n;
   }
