@@ -264,7 +264,8 @@ bool field_step_fused(const pic_ctx* c) {
 // One step from the fields f into o (f.j: the context's current).
 template <typename T>
 pic_status step_fields(pic_ctx* c, const StencilArgs<T>& s, FieldPtrs<T> f, const FieldPtrs<T>& o) {
-  if (c->steps_since_sort >= c->sort_interval) {
+  const bool sparse = particles_sparse(std::is_same<T, double>::value, c->np);   // no bins
+  if (c->steps_since_sort >= c->sort_interval && !sparse) {
     pic_status st = rebin(c);
     if (st != PIC_OK) return st;
   }
@@ -289,7 +290,7 @@ pic_status step_fields(pic_ctx* c, const StencilArgs<T>& s, FieldPtrs<T> f, cons
       CK(c, launch_particle_step<T>(f, bg, c->parts[c->pcur], c->g, s, c->ptile, a, c->bins,
                                     c->stream));
     }
-    if (c->steps_since_sort > c->straggle_after || c->strag_always) {
+    if (!sparse && (c->steps_since_sort > c->straggle_after || c->strag_always)) {
       TimedScope ts(c, 2, 1);
       CK(c, launch_straggler_step<T>(f, bg, c->parts[c->pcur], c->g, s, a, c->bins, c->np,
                                      c->stream));
@@ -310,7 +311,7 @@ pic_status step_fields(pic_ctx* c, const StencilArgs<T>& s, FieldPtrs<T> f, cons
     }
   }
   if (c->timing) c->t_steps++;
-  c->steps_since_sort++;
+  if (c->steps_since_sort < 1 << 30) c->steps_since_sort++;
   return PIC_OK;
 }
 
@@ -872,7 +873,8 @@ pic_status window_after_step(pic_ctx* c) {
 cudaGraphExec_t step_pair_graph(pic_ctx* c) {
   if (c->graphs_off) return nullptr;
   // whether the pair's steps look for particles that left their windows
-  const bool strag = c->np > 0 && c->steps_since_sort + 1 > c->straggle_after;
+  const bool sparse = particles_sparse(c->grid.precision == PIC_FP64, c->np);
+  const bool strag = c->np > 0 && !sparse && c->steps_since_sort + 1 > c->straggle_after;
   for (auto& g : c->sgraph)
     if (g.exec && g.epoch == c->epoch && g.cur == c->cur && g.pcur == c->pcur && g.strag == strag)
       return g.exec;
@@ -922,7 +924,9 @@ pic_status pic_step(pic_ctx* c, int64_t nsteps) {
   while (s < nsteps) {
     // pairs of steps without a re-binning between them replay a captured graph
     // (launch overhead dominates small grids); timing runs take plain launches
-    const int64_t room = std::min<int64_t>(nsteps - s, c->sort_interval - c->steps_since_sort);
+    const bool sparse = particles_sparse(c->grid.precision == PIC_FP64, c->np);   // no re-binning
+    const int64_t room =
+        sparse ? nsteps - s : std::min<int64_t>(nsteps - s, c->sort_interval - c->steps_since_sort);
     if (c->mw_start >= 0 || c->spec) {   // moving window or spectral path: one step at a time
       pic_status st = step_once(c);
       if (st == PIC_OK) st = window_after_step(c);
@@ -936,10 +940,10 @@ pic_status pic_step(pic_ctx* c, int64_t nsteps) {
         // as many pairs as keep the graph's kind (the last ones before a re-binning may
         // have to look for particles that left their windows)
         int64_t pairs = room / 2;
-        if (c->np > 0 && c->steps_since_sort < c->straggle_after)
+        if (c->np > 0 && !sparse && c->steps_since_sort < c->straggle_after)
           pairs = std::min<int64_t>(pairs, (c->straggle_after - c->steps_since_sort + 1) / 2);
         for (int64_t k = 0; k < pairs; ++k) CK(c, cudaGraphLaunch(ex, c->stream));
-        c->steps_since_sort += (int)(2 * pairs);
+        c->steps_since_sort = (int)std::min<int64_t>(c->steps_since_sort + 2 * pairs, 1 << 30);
         c->steps_done += 2 * pairs;
         s += 2 * pairs;
         continue;

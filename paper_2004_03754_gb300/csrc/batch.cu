@@ -108,16 +108,6 @@ __device__ bool grid_wait(const BatchArgs<T>& A, unsigned& epoch) {
   return ok != 0;
 }
 
-// an accumulator at grid nodes offset from the caller's
-template <typename T>
-struct OffsetAcc {
-  GlobAcc<T> a;
-  int o1, o2;
-  __device__ __forceinline__ void add(int l1, int l2, int l3, typename DepositOf<T>::type v) const {
-    a.add(l1 + o1, l2 + o2, l3, v);
-  }
-};
-
 template <typename T>
 __device__ __forceinline__ T* pool_ptr(const BatchArgs<T>& A, int slot, int64_t off) {
   return A.pool + (int64_t)slot * A.total + off;
@@ -205,7 +195,7 @@ __device__ void particle_warp(const BatchArgs<T>& A, const StencilArgs<T>& s, co
     for (int c = 0; c < 3; ++c) {
       ve[c] = SmemView<T>{buf + c * 16, 4, 16, 0};
       vb[c] = SmemView<T>{buf + (3 + c) * 16, 4, 16, 0};
-      acc[c] = OffsetAcc<T>{GlobAcc<T>{run_ptr(A, 12 + c, R), n1, n2, 1, ld}, li[0] - 1, li[1] - 1};
+      acc[c] = OffsetAcc<T>{GlobAcc<T>{run_ptr(A, 12 + c, R), n1, n2, 1, ld}, li[0] - 1, li[1] - 1, 0};
     }
     const int l1[3] = {1, 1, 0}, gc[3] = {li[0], li[1], 0};
     const T f3[3] = {fr[0], fr[1], (T)0};

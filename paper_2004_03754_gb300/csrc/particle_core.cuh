@@ -253,6 +253,16 @@ struct GlobAcc {
   }
 };
 
+// an accumulator at grid nodes offset from the caller's (window-local) ones
+template <typename T>
+struct OffsetAcc {
+  GlobAcc<T> a;
+  int o1, o2, o3;
+  __device__ __forceinline__ void add(int l1, int l2, int l3, typename DepositOf<T>::type v) const {
+    a.add(l1 + o1, l2 + o2, l3 + o3, v);
+  }
+};
+
 // Quadratic B-spline weights around the nearest node, d in [-1/2, 1/2).
 template <typename T>
 PIC_HD void bspline3(T d, T w[3]) {

@@ -348,7 +348,63 @@ __global__ void straggler_kernel(FieldPtrs<T> f, BbarPtrs<T> bg, PartPtrs p, Gri
   }
 }
 
+// Few particles: a warp each, straight from global memory.  The lanes copy the
+// particle's 4^NDIM nodes of E and the time-centred B into shared memory, lane 0
+// advances it from there and deposits into global memory.  No windows, no bins: a
+// tile's window costs the same for one particle as for hundreds.
+template <typename T, int NDIM, bool GAIN>
+__global__ void __launch_bounds__(128) sparse_kernel(FieldPtrs<T> f, BbarPtrs<T> bg, PartPtrs p,
+                                                     GridArgs g, PartArgs a, unsigned* err) {
+  constexpr int NODES = NDIM == 3 ? 64 : 16;
+  __shared__ T sm[4][6 * NODES];
+  const int lane = threadIdx.x & 31;
+  T* buf = sm[threadIdx.x >> 5];
+  const int n1 = g.n[0], n2 = g.n[1], n3 = NDIM == 3 ? g.n[2] : 1;
+  for (int64_t q = blockIdx.x * 4ll + (threadIdx.x >> 5); q < a.np; q += gridDim.x * 4ll) {
+    int gc[3] = {0, 0, 0};
+    T fr[3];
+#pragma unroll
+    for (int d = 0; d < NDIM; ++d) {
+      double frac;
+      gc[d] = floor_split(p.x[d][q] * g.inv_dx[d], frac);
+      fr[d] = to_prec<T>(frac);
+    }
+    const int o3 = NDIM == 3 ? gc[2] - 1 : 0;
+    for (int m = lane; m < NODES; m += 32) {
+      const int64_t r = ((int64_t)wrap_index(o3 + (m >> 4), n3) * n2 + wrap_index(gc[1] - 1 + ((m >> 2) & 3), n2)) *
+                            n1 + wrap_index(gc[0] - 1 + (m & 3), n1);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        buf[c * NODES + m] = f.e[c][r];
+        buf[(3 + c) * NODES + m] = bg.b[c][r];
+      }
+    }
+    __syncwarp();
+    if (lane == 0) {
+      SmemView<T> ve[3], vb[3];
+      OffsetAcc<T> acc[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        ve[c] = SmemView<T>{buf + c * NODES, 4, 16, 0};
+        vb[c] = SmemView<T>{buf + (3 + c) * NODES, 4, 16, 0};
+        acc[c] = OffsetAcc<T>{GlobAcc<T>{f.j[c], n1, n2, n3, n1}, gc[0] - 1, gc[1] - 1, o3};
+      }
+      const int li[3] = {1, 1, NDIM == 3 ? 1 : 0};
+      advance_particle<T, NDIM, -1, GAIN>(ve, vb, acc, p, q, li, fr, gc, g, a, err);
+    }
+    __syncwarp();
+  }
+}
+
 }  // namespace
+
+template <typename T, int NDIM>
+void launch_sparse_nd(const FieldPtrs<T>& f, const BbarPtrs<T>& bg, const PartPtrs& p,
+                      const GridArgs& g, const PartArgs& a, unsigned* err, cudaStream_t st) {
+  const unsigned nb = (unsigned)((a.np + 3) / 4);
+  if (p.wl) sparse_kernel<T, NDIM, true><<<nb, 128, 0, st>>>(f, bg, p, g, a, err);
+  else sparse_kernel<T, NDIM, false><<<nb, 128, 0, st>>>(f, bg, p, g, a, err);
+}
 
 // one CTA per particle tile
 template <typename T, class K>
@@ -383,6 +439,13 @@ cudaError_t launch_particle_step(const FieldPtrs<T>& f, const BbarPtrs<T>& bg, c
                                  const PartArgs& a, const BinBufs& b, cudaStream_t st) {
   const size_t smem = particle_smem_bytes(g.ndim, sizeof(T), t, s.M);
   cudaError_t e;
+  if constexpr (std::is_same<T, double>::value) {
+    if (particles_sparse(true, a.np)) {
+      if (g.ndim == 3) launch_sparse_nd<T, 3>(f, bg, p, g, a, b.err, st);
+      else launch_sparse_nd<T, 2>(f, bg, p, g, a, b.err, st);
+      return cudaGetLastError();
+    }
+  }
   if (g.ndim == 3)
     e = p.wl ? launch_pushers<T, 3, true>(f, bg, p, g, s, t, a, b, smem, st)
              : launch_pushers<T, 3, false>(f, bg, p, g, s, t, a, b, smem, st);

@@ -43,3 +43,35 @@ def test_windows_equal_the_oracle(n, precision, tol):
         L = g.length[d]
         assert np.abs((x[d] - Po.x[d] + L / 2) % L - L / 2).max() <= tol * L, d
     sim.close()
+
+
+@pytest.mark.parametrize("n", [(3, 2), (65, 9), (256, 40), (5, 3, 2), (40, 9, 6)])
+@pytest.mark.parametrize("count", [1, 5, 256, 257])
+@pytest.mark.parametrize("pusher", ["boris", "hc"])
+def test_few_particles_equal_the_oracle(n, count, pusher):
+    # up to 256 particles next to FP64 fields take a warp each, from 257 on tiles
+    from paper_2004_03754_gb300 import pic as P
+    cE, cB = load_table(16, 0.25, 0.3)
+    dx = (inputs.DX1, inputs.DX2, inputs.DX2)[:len(n)]
+    dt = 0.25 * inputs.DX1
+    g = orc.Grid(n, dx, dt, cE, cB)
+    sim = P.Simulation(n, dx, dt, cE, cB, precision="fp64", pusher=pusher)
+    F = orc.Fields(g)
+    for nm, a in zip(NAMES6, inputs.random_fields(g.shape, amp=0.5, seed=17)):
+        getattr(F, nm)[...] = a
+        sim.load_field(nm, a)
+    Ps = inputs.random_particles(n, dx, count, umax=2.0, seed=18)
+    sim.load_particles(Ps.x, Ps.u, Ps.w)
+    Po = orc.Particles(Ps.x, Ps.u, Ps.w)
+    orc.step(g, F, Po, nsteps=25, pusher=pusher)
+    sim.step(25)
+    for nm in NAMES6:
+        ref = getattr(F, nm)
+        assert np.abs(sim.read_field(nm) - ref).max() <= 1e-12 * max(np.abs(ref).max(), 1.0), nm
+    x, u, _ = sim.read_particles()
+    for c in range(3):
+        assert np.abs(u[c] - Po.u[c]).max() <= 1e-11 * np.abs(Po.u[c]).max(), c   # 25 chained pushes
+    for d in range(len(n)):
+        L = g.length[d]
+        assert np.abs((x[d] - Po.x[d] + L / 2) % L - L / 2).max() <= 1e-12 * L, d
+    sim.close()
