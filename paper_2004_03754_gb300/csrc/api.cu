@@ -154,6 +154,46 @@ pic_status build_correction(pic_ctx* c) {
   return PIC_OK;
 }
 
+void free_shares(pic_ctx* c) {
+  pic::TileShares& h = c->bins.share;
+  cudaFree(h.counts);
+  cudaFree(h.list);
+  cudaFree(h.slot);
+  cudaFree(h.scratch);
+  h = pic::TileShares{};
+}
+
+// Lists and scratch for crowded tiles of n particles: shares of a quarter of what an
+// SM gets of all particles (at least 1024, four passes of a CTA), so at most 608 of
+// them.
+pic_status alloc_shares(pic_ctx* c, int64_t n) {
+  pic::TileShares& h = c->bins.share;
+  const int64_t chunk = std::max<int64_t>(1024, (n + 4 * 152 - 1) / (4 * 152));
+  const int most = (int)(n / chunk);
+  h.chunk = 0;
+  if (most == 0) return PIC_OK;   // no tile can be crowded
+  if (h.cap < most) {
+    free_shares(c);
+    h.words = 4 + (particle_window_ints(c->grid.ndim, c->grid.precision == PIC_FP64, c->tsize,
+                                        c->ptile) + 3) / 4 * 4;
+    const size_t bytes = sizeof(int) * (size_t)h.words * most;
+    if (cudaMalloc(&h.counts, 2 * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&h.list, sizeof(pic::TileShare) * most) != cudaSuccess ||
+        cudaMalloc(&h.slot, sizeof(int) * c->ptile.ntiles) != cudaSuccess ||
+        cudaMalloc(&h.scratch, bytes) != cudaSuccess) {
+      cudaGetLastError();   // no room: tiles are not shared
+      free_shares(c);
+      return PIC_OK;
+    }
+    CK(c, cudaMemsetAsync(h.scratch, 0, bytes, c->stream));
+    h.ntiles = c->ptile.ntiles;
+    h.cap = most;
+  }
+  h.most = most;
+  h.chunk = chunk;
+  return PIC_OK;
+}
+
 pic_status alloc_particles(pic_ctx* c, int64_t n) {
   if (n <= c->cap) return PIC_OK;
   for (int s = 0; s < 2; ++s) {
@@ -615,6 +655,7 @@ pic_status pic_destroy(pic_ctx* c) {
   cudaFree(c->bins.strag);
   cudaFree(c->bins.strag_count);
   cudaFree(c->bins.err);
+  free_shares(c);
   for (auto& t : c->tev) {
     cudaEventDestroy(t.second.first);
     cudaEventDestroy(t.second.second);
@@ -718,6 +759,7 @@ pic_status pic_load_particles(pic_ctx* c, int64_t n, const double* x, const doub
   CK(c, cudaSetDevice(c->device));
   const int nd = c->grid.ndim;
   pic_status st = alloc_particles(c, n);
+  if (st == PIC_OK) st = alloc_shares(c, n);
   if (st != PIC_OK) return st;
   ++c->epoch;  // particle buffers and count change: captured step graphs are stale
   c->np = n;

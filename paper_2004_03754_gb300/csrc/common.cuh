@@ -162,6 +162,34 @@ struct PartArgs {
 // warps, two per SM, end before a tile has staged its window.
 __host__ __device__ inline bool particles_sparse(bool f64, int64_t np) { return f64 && np <= 256; }
 
+// Crowded tiles: a tile of more than `chunk` particles is shared by several CTAs (its
+// time would otherwise bound the whole step: an electron sheet in front of a strong
+// pulse put 12 times the mean into one tile).  Each share runs in a current window of
+// its own, on the scales of the whole tile; the windows' integers are added up in
+// `scratch` and the last CTA to arrive flushes the sum, so the current does not depend
+// on the split.  The list is made with the tile counts of each re-binning.  The line
+// is a quarter of what an SM gets of all particles: four tiles of that size are
+// resident on an SM at least in part, so a smaller one does not stand out; and never
+// under 1024 particles, where staging the windows again costs what the split gives.
+// 2D compensated, 1.5 M electrons behind a pulse of a0 = 100, particle kernel per
+// step: largest tile 3.2 k particles 0.75 -> 0.79 ms, 9.4 k 1.18 -> 0.89, 12 k
+// 1.39 -> 0.94; with no crowded tile 1.58 -> 1.56 (33.5 M electrons, mixed) and
+// 2.16 -> 2.16 ms (8.4 M, FP64).
+struct TileShare {
+  int tile, part, slot;
+};
+struct TileShares {
+  int64_t chunk;      // particles per share; 0: no list
+  int64_t ntiles;
+  int* counts;        // [0] shares beyond the first of their tiles, [1] crowded tiles
+  TileShare* list;    // the former
+  int* slot;          // ntiles: index of a crowded tile
+  int* scratch;       // per crowded tile: arrival count (16 bytes), then the window's integers
+  int words;          // ints per crowded tile
+  int most;           // upper bound of both counts: particles / chunk
+  int cap;            // the most that list and scratch hold
+};
+
 struct BinBufs {
   int64_t* count;     // ntiles + 1 (the last bin holds particles being dropped)
   int64_t* start;     // ntiles + 2
@@ -171,6 +199,7 @@ struct BinBufs {
   unsigned long long* strag_count;
   unsigned* err;
   int64_t* part;      // bin_scan_chunks(ntiles + 1): chunk sums of the scan
+  TileShares share{};
 };
 
 // chunks of the tile-count scan for n counts (the size of BinBufs::part)
@@ -208,6 +237,9 @@ cudaError_t launch_renumber(int64_t* id, int64_t np_old, int64_t kept, int64_t* 
 
 // W_LWFA then W_DLA of every particle, in load order, into out (2 np values)
 cudaError_t launch_unpermute_gain(const PartPtrs& p, int64_t np, double* out, cudaStream_t st);
+
+// ints of one tile's current window
+int particle_window_ints(int ndim, bool f64, size_t tsize, const PartTile& t);
 
 size_t particle_smem_bytes(int ndim, size_t tsize, const PartTile& t, int M);
 

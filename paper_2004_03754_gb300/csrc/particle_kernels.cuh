@@ -123,9 +123,32 @@ __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::c
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long wmax_warp[32];
   T* sm = reinterpret_cast<T*>(smem_raw);
-  const unsigned tile = blockIdx.x;
-  const int64_t pbeg = bins.start[tile], pend = bins.start[tile + 1];
-  if (pbeg == pend) return;
+  // CTAs beyond the tiles take the further shares of crowded tiles
+  unsigned tile = blockIdx.x;
+  int part = 0;
+  if (tile >= t.ntiles) {
+    const unsigned x = tile - (unsigned)t.ntiles;
+    if (x >= (unsigned)bins.share.counts[0]) return;
+    const TileShare sh = bins.share.list[x];
+    tile = (unsigned)sh.tile;
+    part = sh.part;
+  }
+  const int64_t tbeg = bins.start[tile], tend = bins.start[tile + 1];
+  if (tbeg == tend) return;
+  int64_t pbeg = tbeg, pend = tend;
+  // (in shared memory: read again after the particle loop, no registers held across it)
+  __shared__ int s_parts, s_slot;
+  if (threadIdx.x == 0) s_parts = 1;
+  if (bins.share.chunk > 0 && tend - tbeg > bins.share.chunk) {
+    const int parts = (int)((tend - tbeg + bins.share.chunk - 1) / bins.share.chunk);
+    const int64_t per = (tend - tbeg + parts - 1) / parts;
+    pbeg = min(tend, tbeg + part * per);
+    pend = min(tend, pbeg + per);
+    if (threadIdx.x == 0) {
+      s_parts = parts;
+      s_slot = bins.share.slot[tile];
+    }
+  }
   prefetch_chunk<NDIM>(p, pbeg, min(pend, pbeg + (int64_t)blockDim.x));
   int tc[3];
   {
@@ -174,7 +197,7 @@ __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::c
   {
     // largest |w| of the tile (non-negative doubles order as their bit patterns)
     unsigned long long wm = 0ull;
-    for (int64_t q = pbeg + threadIdx.x; q < pend; q += blockDim.x)
+    for (int64_t q = tbeg + threadIdx.x; q < tend; q += blockDim.x)
       wm = max(wm, (unsigned long long)__double_as_longlong(p.w[q]) & 0x7fffffffffffffffull);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) wm = max(wm, __shfl_xor_sync(0xffffffffu, wm, o));
@@ -197,8 +220,8 @@ __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::c
     // magnitude: the node sums of the quadratic spline have slope <= 1) times a
     // time-averaged shape weight (<= 1), so at most |w| |v_d| < |w|; the 2D
     // out-of-plane term is w v3 times a path-averaged weight product (<= 1)
-    if constexpr (F64) fix64_scales(pend - pbeg, __longlong_as_double((long long)wm), eS, l64);
-    else fix_scales(pend - pbeg, narrow_signed(__longlong_as_double((long long)wm)) * 1.001f, S, L);
+    if constexpr (F64) fix64_scales(tend - tbeg, __longlong_as_double((long long)wm), eS, l64);
+    else fix_scales(tend - tbeg, narrow_signed(__longlong_as_double((long long)wm)) * 1.001f, S, L);
   }
 
   // views indexed by the current window's node
@@ -266,6 +289,26 @@ __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::c
     advance_particle<T, NDIM, PUSH, GAIN>(ve, vb, acc, p, q, li, fr, gc, g, a, bins.err);
   }
   __syncthreads();
+  if (s_parts > 1) {
+    // add this share's integers to the tile's; the last share takes the sum
+    __shared__ int last;
+    int* scr = bins.share.scratch + (size_t)s_slot * bins.share.words;
+    const int words = (F64 ? 9 : 6) * nW;
+    for (int q = threadIdx.x; q < words; q += blockDim.x)
+      if (sJh[q] != 0) atomicAdd(scr + 4 + q, sJh[q]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(scr, 1) == s_parts - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int q = threadIdx.x; q < words; q += blockDim.x) {
+      sJh[q] = __ldcg(scr + 4 + q);
+      scr[4 + q] = 0;   // for the next step
+    }
+    if (threadIdx.x == 0) scr[0] = 0;
+    __syncthreads();
+  }
   auto flush = [&](auto C) {
     constexpr int c = decltype(C)::value;
     for_window_chunks<c, NDIM>(W, wlo, g, [&](int o, int j, int k, int i) {
@@ -413,7 +456,8 @@ cudaError_t launch_tiles(K kern, const FieldPtrs<T>& f, const BbarPtrs<T>& bg, c
                          const PartArgs& a, const BinBufs& b, size_t smem, int threads, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)t.ntiles, threads, smem, st>>>(f, bg, p, g, s, t, a, b);
+  const unsigned extra = b.share.chunk > 0 ? (unsigned)b.share.most : 0u;
+  kern<<<(unsigned)t.ntiles + extra, threads, smem, st>>>(f, bg, p, g, s, t, a, b);
   return cudaGetLastError();
 }
 

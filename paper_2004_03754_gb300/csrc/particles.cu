@@ -92,6 +92,14 @@ __global__ void __launch_bounds__(kScanT) bin_chunk_out_kernel(BinBufs b, int64_
   for (int k = 0; k < kScanPer; ++k) {
     if (base + k < n) b.start[base + k] = run;
     run += v[k];
+    // shares of a crowded tile beyond its first
+    if (b.share.chunk > 0 && v[k] > b.share.chunk && base + k < b.share.ntiles) {
+      const int parts = (int)((v[k] + b.share.chunk - 1) / b.share.chunk);
+      const int slot = atomicAdd(&b.share.counts[1], 1);
+      const int at = atomicAdd(&b.share.counts[0], parts - 1);
+      b.share.slot[base + k] = slot;
+      for (int p = 1; p < parts; ++p) b.share.list[at + p - 1] = TileShare{(int)(base + k), p, slot};
+    }
   }
   if (base <= n - 1 && n - 1 < base + kScanPer) b.start[n] = run;   // the total
 }
@@ -100,6 +108,7 @@ __global__ void __launch_bounds__(kScanT) bin_chunk_out_kernel(BinBufs b, int64_
 __global__ void __launch_bounds__(1024) bin_part_scan_kernel(BinBufs b, int64_t m) {
   __shared__ int64_t part[1024];
   const int tid = threadIdx.x;
+  if (b.share.chunk > 0 && tid < 2) b.share.counts[tid] = 0;
   const int64_t per = (m + 1023) / 1024;
   const int64_t lo = tid * per, hi = (lo + per < m) ? lo + per : m;
   int64_t s = 0;
@@ -172,6 +181,12 @@ inline int grid_for(int64_t n) {
 }
 
 }  // namespace
+
+int particle_window_ints(int ndim, bool f64, size_t tsize, const PartTile& t) {
+  int nj = 1;
+  for (int d = 0; d < ndim; ++d) nj *= j_window(d, t.t[d], t.g[d], 16 / (int)tsize).w;
+  return (f64 ? 9 : 6) * nj;
+}
 
 size_t particle_smem_bytes(int ndim, size_t tsize, const PartTile& t, int M) {
   (void)M;

@@ -75,3 +75,36 @@ def test_few_particles_equal_the_oracle(n, count, pusher):
         L = g.length[d]
         assert np.abs((x[d] - Po.x[d] + L / 2) % L - L / 2).max() <= 1e-12 * L, d
     sim.close()
+
+
+@pytest.mark.parametrize("n", [(64, 32), (70, 33), (40, 20, 12)])
+@pytest.mark.parametrize("precision, tol", [("fp64", 1e-12), ("mixed", 5e-6), ("compensated", 5e-6)])
+@pytest.mark.parametrize("count", [1024, 1025, 9000])
+def test_crowded_tiles_equal_the_oracle(n, precision, tol, count):
+    # nearly all particles in a few cells: their tiles are shared by several CTAs (from
+    # 1025 particles on), whose windows are added up, step after step
+    from paper_2004_03754_gb300 import pic as P
+    cE, cB = load_table(16, 0.5, 0.3)
+    dx = (inputs.DX1, inputs.DX2, inputs.DX2)[:len(n)]
+    g = orc.Grid(n, dx, inputs.DT, cE, cB)
+    sim = P.Simulation(n, dx, inputs.DT, cE, cB, precision=precision, pusher="boris")
+    F = orc.Fields(g)
+    for nm, a in zip(NAMES6, inputs.random_fields(g.shape, amp=0.5, seed=27)):
+        getattr(F, nm)[...] = a
+        sim.load_field(nm, a)
+    Ps = inputs.random_particles(n, dx, count, umax=2.0, seed=28)
+    for d in range(len(n)):   # the crowd: cells 6 .. 10 of each axis
+        Ps.x[d][: count - 20] = (6 + 4 * Ps.x[d][: count - 20] / (n[d] * dx[d])) * dx[d]
+    Ps.w[:] = -1e-4 * np.linspace(0.2, 1.0, count)
+    sim.load_particles(Ps.x, Ps.u, Ps.w)
+    Po = orc.Particles(Ps.x, Ps.u, Ps.w)
+    for steps in (1, 3):
+        orc.step(g, F, Po, nsteps=steps)
+        sim.step(steps)
+        for nm in NAMES6:
+            ref = getattr(F, nm)
+            assert np.abs(sim.read_field(nm) - ref).max() <= tol * max(np.abs(ref).max(), 0.5), nm
+        x, u, _ = sim.read_particles()
+        for c in range(3):
+            assert np.abs(u[c] - Po.u[c]).max() <= tol * np.abs(Po.u[c]).max(), c
+    sim.close()
