@@ -37,13 +37,6 @@ FP64_FLOP_PER_PUSH = 70   # 2D Boris (58) + gamma (7) + position update (5), FMA
 # (16 subtractions + 16 FMA = 48 FLOP each) plus the Yee differences, current term and updates
 FIELD_FLOP_PER_CELL = {2: 214, 3: 226}
 FP64_PEAK_TFLOPS_AT_MAX = 304 * 2 * 2070e6 / 1e12   # 304 DFMA/cycle/GPU at 2070 MHz
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch from ncu, per
-# push: the particle kernel on the 2048x512 workload (python bench.py --small, launch 4),
-# scaled to the bench workload's launch (traffic grows with the particles)
-PARTICLE_KERNEL_TRAFFIC_PER_PUSH = (366.734592e6 + 240.926464e6) / 6295552
-TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch: particle "
-                  "kernel on the 2048x512 case (6,295,552 electrons) scaled by the particles to "
-                  "this launch")
 WORKLOAD = "2D 4096x1024 plasma 8ppc a0=4, customised M=16 solver, Boris"
 
 
@@ -229,17 +222,15 @@ def run_gpu(args):
     value = whole_job_rate(npart, steps, world, ms_local)
     cells_s = whole_job_rate(ncell, steps, world, ms_local)
     t = mixed["timing"]
-    # roofline of the dominant kernel (particles).  Its binding resource is the
-    # FP64 pipe (GB300: 2 DFMA/clk/SM): algorithmic FP64 work per push is the
-    # Boris rotation, gamma and the position update, 70 FLOP (FMA = 2).  The
-    # HBM view (88 algorithmic bytes per push) is reported beside it.
+    # roofline of the dominant kernel (particles), 88 algorithmic bytes per push
+    # against HBM.  What binds it is warp issue (74 % of the slots) and the shared-memory
+    # pipe (61 %): the push runs in FP32 pairs, so the FP64 pipe holds little work.
     part_ms = t.ms_particles / steps
     alg_bytes = 88.0 * npart
     peak, peak_kind = measured_peaks()
     achieved = alg_bytes / (part_ms / 1e3) / 1e9
     sm_mhz = (mixed["clocks"] or {}).get("sm_mhz") or 2070.0
     fp64_peak = 304 * 2 * sm_mhz * 1e6 / 1e12          # TFLOP/s at the sampled clock
-    fp64_ach = FP64_FLOP_PER_PUSH * npart / (part_ms / 1e3) / 1e12
     fld_ms = t.ms_fields / steps
     fld_gbs = 60.0 * ncell / (fld_ms / 1e3) / 1e9
     sim = mixed["sim"]
@@ -341,22 +332,17 @@ def run_gpu(args):
         "kernel_ms_per_step": {"rebin": t.ms_rebin / steps, "particles": part_ms,
                                "stragglers": t.ms_stragglers / steps,
                                "correction": t.ms_correction / steps, "fields": fld_ms},
-        "roofline": {"bound": "alu", "kernel": "particle_kernel<float,2>",
-                     "achieved": fp64_ach, "peak": fp64_peak, "unit": "TFLOP/s (FP64)",
-                     "frac": fp64_ach / fp64_peak,
-                     "traffic": PARTICLE_KERNEL_TRAFFIC_PER_PUSH * npart,
-                     "traffic_source": TRAFFIC_SOURCE,
-                     "alg_flop_per_launch": FP64_FLOP_PER_PUSH * npart,
-                     "peak_derivation": "304 DFMA/cycle/GPU x 2 FLOP x sampled SM clock",
-                     "hbm_view": {"achieved": achieved, "peak": peak, "unit": "GB/s",
-                                  "frac": achieved / peak, "peak_kind": peak_kind,
-                                  "alg_bytes_per_launch": alg_bytes}},
-        "field_kernel_roofline": {"bound": "hbm", "kernel": "field_march_kernel<float,16>",
+        "roofline": {"bound": "hbm", "kernel": "particle_kernel<float,2>",
+                     "achieved": achieved, "peak": peak, "unit": "GB/s",
+                     "frac": achieved / peak, "peak_kind": peak_kind,
+                     "alg_bytes_per_launch": alg_bytes, "traffic": None,
+                     "traffic_source": "not captured for the bench workload",
+                     "binding": "warp issue 74 %, shared-memory pipe 61 % (ncu, 2048x512 case)"},
+        "field_kernel_roofline": {"bound": "hbm", "kernel": "faraday_rows_kernel + ampere_rows_kernel",
                                   "achieved": fld_gbs, "peak": peak, "unit": "GB/s",
                                   "frac": fld_gbs / peak, "alg_bytes_per_cell": 60,
                                   "traffic": None,
-                                  "traffic_source": "not captured for the current field kernel "
-                                                    "(J read into registers since the last capture)"},
+                                  "traffic_source": "not captured for the bench workload"},
         "fp64_plain": fp64,
         "compensated": comp,
         "ensemble": ensemble,

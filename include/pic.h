@@ -281,8 +281,11 @@ pic_status pic_get_info(pic_ctx* ctx, pic_info* info);
  * depend on it: particles outside their tile's window take a global path. */
 pic_status pic_set_sort_interval(pic_ctx* ctx, int interval);
 
-/* Field tile of the fused Faraday + Ampere kernel (App. B Eqs. (B.1)-(B.2)):
- * t1 x t2 (x t3) cells, x1 fastest; 2D grids need t3 = 1; threads (128, 256 or
+/* By default the field step runs as a Faraday and an Ampere pass over whole rows,
+ * except for large 2D FP32 grids without particles.  This call and
+ * pic_set_field_strip choose the fused Faraday + Ampere kernel and its shape.
+ *
+ * Field tile of that kernel (App. B Eqs. (B.1)-(B.2)): t1 x t2 (x t3) cells, x1 fastest; 2D grids need t3 = 1; threads (128, 256 or
  * 512) per CTA.  staging = 0 lets the kernel stream rows per warp (below) or
  * tiles into shared memory with asynchronous bulk copies where the row pitch
  * allows (n1 and t1 multiples of 16 bytes) and falls back to plain loads
@@ -323,7 +326,7 @@ typedef struct {
   double ms_particles;  /* gather + push + deposit (tiled kernel) */
   double ms_stragglers; /* global-path particles */
   double ms_correction; /* x1 current correction */
-  double ms_fields;     /* fused Faraday + Ampere */
+  double ms_fields;     /* Faraday and Ampere */
   int64_t launches;     /* libpic kernels launched while timing was enabled */
   int64_t steps;        /* steps timed */
 } pic_timing;

@@ -173,8 +173,8 @@ __host__ __device__ inline bool particles_sparse(bool f64, int64_t np) { return 
 // under 1024 particles, where staging the windows again costs what the split gives.
 // 2D compensated, 1.5 M electrons behind a pulse of a0 = 100, particle kernel per
 // step: largest tile 3.2 k particles 0.75 -> 0.79 ms, 9.4 k 1.18 -> 0.89, 12 k
-// 1.39 -> 0.94; with no crowded tile 1.58 -> 1.56 (33.5 M electrons, mixed) and
-// 2.16 -> 2.16 ms (8.4 M, FP64).
+// 1.39 -> 0.94; with no crowded tile 1.58 -> 1.56 (29.4 M electrons, mixed) and
+// 2.16 -> 2.16 ms (6.3 M, FP64).
 struct TileShare {
   int tile, part, slot;
 };
