@@ -613,8 +613,9 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
     ACK(c, P.get(&ckx[s], 2 * n));
     ACK(c, P.get(&cku[s], 3 * n));
   }
-  double *segF, *segx, *segu, *lu, *lx, *wz, *acc, *uend, *xend;
-  ACK(c, P.get(&segF, (size_t)seg * 6 * nc));
+  FieldStates<double> segF{nullptr, FieldStates<double>::pitch_of(nc)};
+  double *segx, *segu, *lu, *lx, *wz, *acc, *uend, *xend;
+  ACK(c, P.get(&segF.base, (size_t)seg * 6 * segF.pitch));
   ACK(c, P.get(&segx, (size_t)seg * 2 * n));
   ACK(c, P.get(&segu, (size_t)seg * 3 * n));
   ACK(c, P.get(&lu, 3 * n));
@@ -660,7 +661,7 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
   }
   const double qm = c->qm;
   auto state = [&](int64_t k, double** f) {   // field state k of the segment in memory
-    for (int m = 0; m < 6; ++m) f[m] = segF + ((size_t)k * 6 + m) * nc;
+    for (int m = 0; m < 6; ++m) f[m] = segF.at(k, m);
   };
   // the steps of one segment from its field state 0, the field states 0 .. steps-1 and
   // the particles of every step kept; the last step goes into `last` (null: not taken)
@@ -733,7 +734,7 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
       a = 1 - a;
       // particles at step k
       AdjPart A;
-      for (int m = 0; m < 6; ++m) A.F[m] = segF + ((size_t)(k - n0) * 6 + m) * nc;
+      for (int m = 0; m < 6; ++m) A.F[m] = segF.at(k - n0, m);
       A.x = segx + (size_t)(k - n0) * 2 * n;
       A.u = segu + (size_t)(k - n0) * 3 * n;
       A.lu = lu;

@@ -95,7 +95,8 @@ cudaError_t launch_field_step(const FieldPtrs<T>& f, const FieldPtrs<T>& out, co
 // The field step as two passes (field_halves.cu): Faraday of f into out.b -- with
 // bg (nullable) also the time-centred B into bg, zeros into f.j and into
 // *strag_count -- and Ampere of f.e and out.b into out.e with the current f.j (null
-// pointers: none).
+// pointers: none).  Every array starts on a 16-byte boundary (the rows are loaded and
+// stored 16 bytes at a time from there); cudaErrorInvalidValue otherwise.
 template <typename T>
 cudaError_t launch_faraday(const FieldPtrs<T>& f, const FieldPtrs<T>& out, const BbarPtrs<T>* bg,
                            const GridArgs& g, const StencilArgs<T>& s,
@@ -103,6 +104,16 @@ cudaError_t launch_faraday(const FieldPtrs<T>& f, const FieldPtrs<T>& out, const
 template <typename T>
 cudaError_t launch_ampere(const FieldPtrs<T>& f, const FieldPtrs<T>& out, const GridArgs& g,
                           const StencilArgs<T>& s, cudaStream_t st);
+
+// Field states E1 E2 E3 B1 B2 B3 of ncell values each, one after another in one
+// allocation: every component starts on a 256-byte boundary, also where ncell is odd.
+template <typename T>
+struct FieldStates {
+  T* base;
+  int64_t pitch;
+  static int64_t pitch_of(int64_t ncell) { return (ncell + 31) / 32 * 32; }
+  T* at(int64_t state, int comp) const { return base + (state * 6 + comp) * pitch; }
+};
 
 template <typename T>
 cudaError_t launch_bbar(const FieldPtrs<T>& f, const GridArgs& g, const StencilArgs<T>& s,

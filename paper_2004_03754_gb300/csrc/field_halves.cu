@@ -27,6 +27,7 @@
 // 128 -> 44 us (all kernels), FP64 2048x512 583 -> 309, compensated 282 -> 64 us, FP32
 // 1501x389 (rows off 16 bytes, CTA tiles before) 72 -> 15 us.
 #include <algorithm>
+#include <initializer_list>
 
 #include "common.cuh"
 #include "field_tile.cuh"
@@ -284,12 +285,24 @@ cudaError_t ampere_mt(const FieldPtrs<T>& f, const FieldPtrs<T>& o, const GridAr
   return cudaGetLastError();
 }
 
+// every array that is given starts on a 16-byte boundary
+template <typename T>
+bool on_16(const FieldPtrs<T>& f, const FieldPtrs<T>& o, const BbarPtrs<T>* bg) {
+  uintptr_t any = 0;
+  for (int c = 0; c < 3; ++c) {
+    for (const T* p : {f.e[c], f.b[c], f.j[c], o.e[c], o.b[c]}) any |= reinterpret_cast<uintptr_t>(p);
+    if (bg) any |= reinterpret_cast<uintptr_t>(bg->b[c]);
+  }
+  return (any & 15u) == 0;
+}
+
 }  // namespace
 
 template <typename T>
 cudaError_t launch_faraday(const FieldPtrs<T>& f, const FieldPtrs<T>& o, const BbarPtrs<T>* bg,
                            const GridArgs& g, const StencilArgs<T>& s, unsigned long long* strag,
                            cudaStream_t st) {
+  if (!on_16(f, o, bg)) return cudaErrorInvalidValue;
   const int mt = stencil_mt(s.M);
   if (g.ndim == 3)
     return mt == 8    ? faraday_mt<T, 3, 8>(f, o, bg, g, s, strag, st)
@@ -303,6 +316,7 @@ cudaError_t launch_faraday(const FieldPtrs<T>& f, const FieldPtrs<T>& o, const B
 template <typename T>
 cudaError_t launch_ampere(const FieldPtrs<T>& f, const FieldPtrs<T>& o, const GridArgs& g,
                           const StencilArgs<T>& s, cudaStream_t st) {
+  if (!on_16(f, o, static_cast<const BbarPtrs<T>*>(nullptr))) return cudaErrorInvalidValue;
   const int mt = stencil_mt(s.M);
   if (g.ndim == 3)
     return mt == 8    ? ampere_mt<T, 3, 8>(f, o, g, s, st)
