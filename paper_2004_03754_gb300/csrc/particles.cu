@@ -27,7 +27,11 @@ __global__ void bin_count_kernel(PartPtrs p, GridArgs g, PartTile t, BinBufs b, 
     for (int d = 0; d < g.ndim; ++d) {
       int c = floor_pos(p.x[d][q] * g.inv_dx[d]);
       if (d == 0) c0 = c;
-      c = c >= g.n[d] ? g.n[d] - 1 : c;
+      // x in the last place below the box's end can round to cell n: the node there
+      // is node 0, so it is binned with the particles of cell 0, whose tile the
+      // particle kernel unwraps cell n into (its window holds both neighbourhoods).
+      // (unsigned: no cell that a position outside the box gives reaches past the bins)
+      c = (unsigned)c >= (unsigned)g.n[d] ? 0 : c;
       tc[d] = c / t.t[d];
     }
     int key = (tc[2] * t.nt[1] + tc[1]) * t.nt[0] + tc[0];
