@@ -272,53 +272,93 @@ struct PairMove {
   float dtig, ig, u[3];   // dt/gamma, 1/gamma, u^{n+1/2}
 };
 
-PIC_HDI bool analytic_push_wide(double qm, double dt, const float eb[6], double u[3]);
+PIC_HDI bool push_wide(double qm, double dt, int kind, const float eb[6], double u[3]);
+
+// max |v_d| below 2^e (e > 0), false for NaN; on the integer pipe
+PIC_HD bool pr_below(const double v[3], int e) {
+  const uint32_t m = 0x7fffffffu;
+  const uint32_t a = (uint32_t)(f64_bits(v[0]) >> 32) & m, b = (uint32_t)(f64_bits(v[1]) >> 32) & m,
+                 c = (uint32_t)(f64_bits(v[2]) >> 32) & m;
+  const uint32_t ab = a > b ? a : b;
+  return (ab > c ? ab : c) < (uint32_t)(1023 + e) << 20;
+}
 
 template <int PUSH, int NDIM>
 PIC_HD bool push_pair(double qm, double dt, int pusher, const float eb[6], double u[3], PairMove& mv) {
-  dfl U[3], du[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) U[d] = pr_split(u[d]);
+  // The pairs hold |u| and |q/m dt E|, |q/m dt B| below 2^28 (gamma^4 within FP32 in the
+  // Higuera-Cary root); anything else, infinities and NaN among it, takes the FP64
+  // push, which either moves the particle or gives a non-finite dt/gamma.
   const int kind = PUSH < 0 ? pusher : PUSH;
-  bool wide = false;
-  if (kind == PIC_ANALYTIC) {
-    wide = !analytic_push_pair(pr_split(qm * dt), eb, U, du);
-  } else if (kind == PIC_HC) {
-    hc_push_pair(pr_split(0.5 * qm * dt), eb, U, du);
-  } else {
-    boris_push_pair(pr_split(0.5 * qm * dt), eb, U, du);
+  const float k = fabsf(narrow_sat(qm * dt));
+  float em = 0.0f;
+  bool inside = pr_below(u, 28);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    em = fmaxf(em, fabsf(eb[c]));
+    inside = inside && eb[c] == eb[c];
   }
-  if (wide) {
-    if (!analytic_push_wide(qm, dt, eb, u)) return false;
+  inside = inside && k * em < 0x1p28f;
+  double un[3] = {u[0], u[1], u[2]};
+  if (inside) {
+    dfl U[3], du[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) U[d] = pr_split(u[d]);
-  } else {
+    if (kind == PIC_ANALYTIC) {
+      inside = analytic_push_pair(pr_split(qm * dt), eb, U, du);
+    } else if (kind == PIC_HC) {
+      hc_push_pair(pr_split(0.5 * qm * dt), eb, U, du);
+    } else {
+      boris_push_pair(pr_split(0.5 * qm * dt), eb, U, du);
+    }
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      u[d] += pr_join(du[d]);
-      U[d] = pr_add(U[d], du[d]);
+    for (int d = 0; d < 3; ++d) un[d] += pr_join(du[d]);
+    inside = inside && pr_below(un, 60);
+    if (inside) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        u[d] = un[d];
+        U[d] = pr_add(U[d], du[d]);
+      }
+      const dfl ig = pr_rsqrt(pr_one_plus_sqr(U));
+      const dfl dtig = pr_norm(pr_mul(pr_split(dt), ig));
+#pragma unroll
+      for (int d = 0; d < NDIM; ++d) mv.dx[d] = pr_mul(dtig, U[d]);
+      mv.dtig = dtig.hi;
+      mv.ig = ig.hi;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) mv.u[d] = U[d].hi;
+      return true;
     }
   }
-  const dfl ig = pr_rsqrt(pr_one_plus_sqr(U));
-  const dfl dtig = pr_norm(pr_mul(pr_split(dt), ig));
+  if (!push_wide(qm, dt, kind, eb, u)) return false;
+  const double ig = rsqrt_nr<1>(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+  const double dtig = dt * ig;
+  // (a non-finite dt/gamma must reach the caller's check as such)
+  mv.dtig = isfinite(dtig) ? narrow_signed(dtig) : NAN;
+  mv.ig = narrow_signed(ig);
 #pragma unroll
-  for (int d = 0; d < NDIM; ++d) mv.dx[d] = pr_mul(dtig, U[d]);
-  mv.dtig = dtig.hi;
-  mv.ig = ig.hi;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) mv.u[d] = U[d].hi;
+  for (int d = 0; d < 3; ++d) {
+    if (d < NDIM) mv.dx[d] = pr_split(dtig * u[d]);
+    mv.u[d] = narrow_signed(u[d]);
+  }
   return true;
 }
 
-// the FP64 analytic push of FP32 fields (strong fields; out of line)
+// the FP64 push of a particle in FP32 fields (out of line)
 #ifdef __CUDA_ARCH__
 __noinline__
 #endif
-PIC_HDI bool analytic_push_wide(double qm, double dt, const float eb[6], double u[3]) {
+PIC_HDI bool push_wide(double qm, double dt, int kind, const float eb[6], double u[3]) {
   double e[6];
-  for (int c = 0; c < 6; ++c) e[c] = widen(eb[c]);
+  for (int c = 0; c < 6; ++c) e[c] = (double)eb[c];
   double v[3] = {u[0], u[1], u[2]};
-  if (analytic_push_series(qm, dt, e, v) < 0) return false;
+  if (kind == PIC_ANALYTIC) {
+    if (analytic_push_series(qm, dt, e, v) < 0) return false;
+  } else if (kind == PIC_HC) {
+    hc_push<1>(qm, dt, e, v);
+  } else {
+    boris_push<1>(qm, dt, e, v);
+  }
   for (int d = 0; d < 3; ++d) u[d] = v[d];
   return true;
 }
