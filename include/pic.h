@@ -62,8 +62,10 @@ typedef enum {
 /* precision:
  *   PIC_FP64         every field and particle quantity in FP64;
  *   PIC_MIXED        fields, gather and deposit in FP32, momentum/gamma/positions FP64
- *                    (field error ~6e-8 relative per value; the single-electron
- *                    energy leaves 1e-4 of FP64 beyond a0 ~ 10, see below);
+ *                    (in pic_step the rotation of the Boris and Higuera-Cary pushers and
+ *                    the higher orders of the analytic one in FP32 pairs where that is
+ *                    as close to 64 bits; field error ~6e-8 relative per value; the
+ *                    single-electron energy leaves 1e-4 of FP64 beyond a0 ~ 10, see below);
  *   PIC_COMPENSATED  E and B stored and updated as FP32 pairs hi + lo (48-bit
  *                    significand, FP32 error-free arithmetic, 8 bytes per value),
  *                    gather in that arithmetic, push and positions FP64, current

@@ -62,12 +62,12 @@ constexpr AnTerms as_terms_table(double tol) {
   }
   return t;
 }
-// FP64 series (2^-60), FP32-pair series (2^-50), FP32 series (2^-27); the
-// coefficients in FP64 and as FP32 pairs
+// FP64 series (2^-60) and FP32 series (2^-27); the coefficients in FP64 and as FP32
+// pairs
 struct AsTables {
   AnCoef c;
   float h2[21], l2[21], h3[21], l3[21];
-  AnTerms t64, t48, t24;
+  AnTerms t64, t24;
 };
 constexpr AsTables as_tables() {
   AsTables t{};
@@ -81,7 +81,6 @@ constexpr AsTables as_tables() {
     }
   }
   t.t64 = as_terms_table(8.7e-19);
-  t.t48 = as_terms_table(8.9e-16);
   t.t24 = as_terms_table(7.5e-9);
   return t;
 }

@@ -324,7 +324,7 @@ pic_status step_fields(pic_ctx* c, const StencilArgs<T>& s, FieldPtrs<T> f, cons
     CK(c, launch_faraday<T>(f, o, parts ? &bg : nullptr, c->g, s, c->bins.strag_count, c->stream));
   }
   if (parts) {
-    PartArgs a{c->qm, c->grid.pusher, c->np};
+    const PartArgs a = part_args(c->qm, c->dt, c->grid.pusher, c->np);
     {
       TimedScope ts(c, 1, 1);
       CK(c, launch_particle_step<T>(f, bg, c->parts[c->pcur], c->g, s, c->ptile, a, c->bins,
@@ -814,7 +814,7 @@ pic_status one_step_spectral(pic_ctx* c) {
   }
   if (c->np > 0) {
     CK(c, cudaMemsetAsync(c->bins.strag_count, 0, sizeof(unsigned long long), c->stream));
-    PartArgs a{c->qm, c->grid.pusher, c->np};
+    const PartArgs a = part_args(c->qm, c->dt, c->grid.pusher, c->np);
     BbarPtrs<double> bg{{bb[0], bb[1], bb[2]}};
     {
       TimedScope ts(c, 1, 1);

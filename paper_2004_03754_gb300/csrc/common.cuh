@@ -10,6 +10,7 @@
 
 #include "march_layout.cuh"
 #include "pic.h"
+#include "push_const.h"
 
 namespace pic {
 
@@ -165,7 +166,11 @@ struct PartArgs {
   double qm;
   int pusher;
   int64_t np;
+  PushConst push{};   // of the push next to FP32 fields (zeros: its FP64 form)
 };
+inline PartArgs part_args(double qm, double dt, int pusher, int64_t np) {
+  return PartArgs{qm, pusher, np, push_const(qm, dt)};
+}
 
 // Few enough particles to take a warp each instead of tiles (FP64 fields; FP32 currents
 // keep their windows, whose sums are rounded once): 512x128 cells with one electron, 20

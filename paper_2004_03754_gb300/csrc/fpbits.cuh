@@ -158,6 +158,23 @@ PIC_HD int floor_split(double c, double& frac) {
   return e < 0 ? 0 : (int)(m >> sh);
 }
 
+// the same with the fraction rounded to FP32 (as narrow_signed of it), no FP64 operation
+PIC_HD int floor_split(double c, float& frac) {
+  const uint64_t b = f64_bits(c);
+  const int e = (int)((int64_t)b >> 52) - 1023;
+  const uint64_t m = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+  const int s = e < 0 ? 0 : (e > 52 ? 52 : e);
+  const uint64_t y = b << 12 << s;           // the fraction in units of 2^-64
+  // (1.mantissa 2^e below one: y would lose the leading bit)
+#ifdef __CUDA_ARCH__
+  const float f = __ull2float_rn(y);
+#else
+  const float f = (float)y;
+#endif
+  frac = e < 0 ? narrow_signed(c) : f * 5.42101086242752217e-20f;   // 2^-64
+  return e < 0 ? 0 : (int)(m >> (52 - s));
+}
+
 // floor(c) for c in [0, 2^31) by the mantissa shift alone (integer pipe)
 PIC_HD int floor_pos(double c) {
   const int64_t b = (int64_t)f64_bits(c);

@@ -1,32 +1,52 @@
-// pair_push.cuh -- the momentum advance of particles in FP32 fields, in FP32 pairs
-// (dfloat.cuh: hi + lo, about 47 bits) added to the FP64 momentum and position.
+// pair_push.cuh -- the push of particles in FP32 fields: the FP64 push of pushers.cuh
+// with the parts that lose nothing by it in FP32 pairs (dfloat.cuh: hi + lo, 48 bits).
 //
-// Why: FP64 instructions issue at 1/64 of the FP32 rate on this GPU, and the FP64
-// Boris push of 49 of them kept that pipe 83 % busy and the rest of the SM idle.
-// With FP32 fields (relative rounding 6e-8) a push needs far fewer than 53 bits in
-// its *change* of u: u^{n+1/2} = u^{n-1/2} + du and x^{n+1} = x^n + dx are added in
-// FP64, so nothing of the state is rounded to the pairs' width, and du, dx come
-// from error-free FP32 transformations with a relative error near 2^-45 (the FP64
-// form with one Newton step of its reciprocals had 2^-43).  An FP64 operation
-// takes the issue slots of 64 FP32 ones here; its pair form takes 4 to 11.
-// Measured (one step, particle kernel): 2D Boris, 29.4 M electrons 2.61 -> 2.02 ms;
-// 2D Higuera-Cary, 1.4 M electrons 0.280 -> 0.118 ms; 3D analytic, 84 M electrons
-// 29.2 -> 24.6 ms (there the windows' handling is half of what remains).
+// Why: FP64 instructions issue at 1/64 of the FP32 rate on this GPU, and the FP64 Boris
+// push of 49 of them kept that pipe 83 % busy and the rest of the SM idle.  In pairs
+// are only changes of u that are small against u, or that the FP64 form next to FP32
+// fields leaves less accurate (one Newton step per reciprocal, 2^-44):
+//   Boris, Higuera-Cary   the rotation about B, while |t| = |h B|/gamma < 1/4;
+//   analytic              what L^2 and higher powers add to U + s L U, while the
+//                         arguments of the exponential are below 1/8.
+// The electric kicks, s L U, the residual of the proper time, gamma and the move
+// (dt/gamma) u stay in FP64.  Every other particle, infinities, NaN and momenta past
+// 2^40 among them, takes the FP64 push.  34 -> 22 FP64 instructions per 2D Boris push
+// against the FP64 form with its cells; 3D analytic 153 -> 66.
+//
+// Error against 64 bits (113-bit reference on the device, 5e5 electrons in pulses of
+// a0 = 1 to 100 with plasma fields, at rest to gamma = 600): |du|/|u| root mean square
+// and 99th percentile, the FP64 form before the arrow
+//   Boris 3.8e-16 -> 3.4e-16, 1.3e-15 -> 1.1e-15;  Higuera-Cary 2.0e-15 -> 3.3e-16,
+//   6.2e-15 -> 1.2e-15;  analytic 1.1e-16 -> 8.1e-17, 2.5e-16 -> 1.8e-16;
+// the move 3.2e-15 dt in all (the reciprocal's one Newton step).
+// Measured: 2D Boris, 29.4 M electrons, ten steps and their read-back, all FP64 rotation
+// and cells 24.2 -> 20.2 ms; 2D Higuera-Cary, 1.4 M, twelve steps 2.80 -> 2.24 ms; 3D
+// analytic, 84 M, two steps 54.8 -> 42.1 ms.
 //
 // Products feeding a TwoSum are rounded on their own (mul_rn); sums written
 // plainly hold no product, so no contraction can break them.
 #pragma once
 #include "dfloat.cuh"
 #include "analytic_series.cuh"
+#include "push_const.h"
 #include "pushers.cuh"
 
 namespace pic {
+
+// nearest integer, |x| < 2^31
+PIC_HD int32_t round_int(float x) {
+#ifdef __CUDA_ARCH__
+  return __float2int_rn(x);
+#else
+  return (int32_t)nearbyintf(x);
+#endif
+}
 
 // ---- pair arithmetic without renormalisation where the next operation allows it
 
 // x = hi + lo: hi the FP32 value nearest to x, lo the rest rounded to FP32
 // (relative error below 2^-49), on the integer pipe.  |x| < 2^-126 gives zero,
-// |x| < 2^-74 no low part.
+// |x| < 2^-74 no low part; |x| < 2^128.
 PIC_HD dfl pr_split(double x) {
   const uint64_t b = f64_bits(x);
   const uint64_t mag = b & 0x7fffffffffffffffull;
@@ -41,8 +61,18 @@ PIC_HD dfl pr_split(double x) {
   const float l = mul_rn((float)d, f32_from_bits(sc));
   return dfl(f32_from_bits(h | sign), f32_from_bits(f32_bits(l) ^ sign));
 }
-// the pair in FP64 (exact unless a part is subnormal)
-PIC_HD double pr_join(dfl a) { return widen_normal(a.hi) + widen_normal(a.lo); }
+// the pair in FP64, rounded once, |lo| < 2^-21 |hi|: lo enters hi's FP64 mantissa as an
+// integer (the integer pipe; below 2^-74, where its scale leaves FP32, an FP64 add)
+PIC_HD double pr_join(dfl a) {
+  const uint32_t h = f32_bits(a.hi), mag = h & 0x7fffffffu, eh = mag & 0x7f800000u;
+  if (eh <= (52u << 23)) return widen_normal(a.hi) + widen_normal(a.lo);
+  // lo in units of hi's FP64 last place (half of that below a power of two), signed as hi
+  const bool down = (mag & 0x007fffffu) == 0u && ((f32_bits(a.lo) ^ h) >> 31) != 0u;
+  const float unit = f32_from_bits((306u << 23) - eh + (down ? 1u << 23 : 0u));   // 2^(52 - e)
+  const int32_t d = round_int(mul_rn(a.lo, f32_from_bits(f32_bits(unit) ^ (h & 0x80000000u))));
+  const uint64_t m = ((uint64_t)((mag >> 3) + 0x38000000u) << 32 | (uint64_t)(mag << 29)) + (uint64_t)(int64_t)d;
+  return f64_from_bits(m | (uint64_t)(h & 0x80000000u) << 32);
+}
 
 PIC_HD dfl pr_mul(dfl a, dfl b) {
   const float p = mul_rn(a.hi, b.hi);
@@ -69,22 +99,20 @@ PIC_HD dfl pr_sqr(dfl a) {
 }
 // a + b, the low part not renormalised
 PIC_HD dfl pr_add_raw(dfl a, dfl b) {
-  const dfl s = two_sum(a.hi, b.hi);
+  const dfl s = dfl::two_sum(a.hi, b.hi);
   return dfl(s.hi, s.lo + (a.lo + b.lo));
 }
-PIC_HD dfl pr_norm(dfl a) { return fast_two_sum(a.hi, a.lo); }
+PIC_HD dfl pr_norm(dfl a) { return dfl::fast_two_sum(a.hi, a.lo); }
 PIC_HD dfl pr_add(dfl a, dfl b) { return pr_norm(pr_add_raw(a, b)); }
 PIC_HD dfl pr_neg(dfl a) { return dfl(-a.hi, -a.lo); }
-// a b - c d
-PIC_HD dfl pr_det(dfl a, dfl b, dfl c, dfl d) { return pr_add_raw(pr_mul(a, b), pr_neg(pr_mul(c, d))); }
-// 1 + |v|^2 (all terms positive: each TwoSum may take the larger sum first)
-PIC_HD dfl pr_one_plus_sqr(const dfl v[3]) {
-  dfl s(1.0f, 0.0f);
-#pragma unroll
-  for (int d = 0; d < 3; ++d) s = pr_add_raw(s, pr_sqr(v[d]));
-  return pr_norm(s);
+// v . b and component a x b of v x b, b in FP32
+PIC_HD dfl pr_dotf(const dfl v[3], const float b[3]) {
+  return pr_norm(pr_add_raw(pr_add_raw(pr_mulf(v[0], b[0]), pr_mulf(v[1], b[1])), pr_mulf(v[2], b[2])));
 }
-// 1/sqrt(x), 1/x, x >= 1 (positive normal), x normalised: the FP32 seed and one
+PIC_HD dfl pr_crossf(const dfl v[3], const float b[3], int i, int j) {
+  return pr_norm(pr_add_raw(pr_mulf(v[i], b[j]), pr_mulf(v[j], -b[i])));
+}
+// 1/sqrt(x), 1/x, x positive normal and normalised: the FP32 seed and one
 // Newton step whose residual is formed exactly, with the next term of its series
 PIC_HD dfl pr_rsqrt(dfl x) {
   const float y = seed_rsqrt(x.hi);
@@ -93,274 +121,264 @@ PIC_HD dfl pr_rsqrt(dfl x) {
   float r = (1.0f - p) - fmaf(x.hi, s.hi, -p);       // 1 - x y^2
   r = fmaf(-x.hi, s.lo, r);
   r = fmaf(-x.lo, s.hi, r);
-  return fast_two_sum(y, mul_rn(y, fmaf(mul_rn(0.375f, r), r, 0.5f * r)));
+  return dfl::fast_two_sum(y, mul_rn(y, fmaf(mul_rn(0.375f, r), r, 0.5f * r)));
 }
 PIC_HD dfl pr_rcp(dfl x) {
   const float y = seed_rcp(x.hi);
   float r = fmaf(-x.hi, y, 1.0f);
   r = fmaf(-x.lo, y, r);
-  return fast_two_sum(y, mul_rn(y, fmaf(r, r, r)));
+  return dfl::fast_two_sum(y, mul_rn(y, fmaf(r, r, r)));
 }
 
-// ---- Boris: du = (u- + u- x t) x s + 2 h E with u- = u + h E, h = q dt/2m
-PIC_HD void boris_push_pair(dfl h, const float eb[6], const dfl u[3], dfl du[3]) {
-  dfl k[3], m[3], t[3], v[3];
+// The leading word of |x| (orders as |x|; infinities and NaN are the largest)
+PIC_HD uint32_t mag_word(double x) { return (uint32_t)(f64_bits(x) >> 32) & 0x7fffffffu; }
+PIC_HD bool mag_sign(double x) { return (f64_bits(x) >> 63) != 0; }
+constexpr uint32_t mag_word_of(int e) { return (uint32_t)(1023 + e) << 20; }   // that of 2^e
+
+// 1 + |v|^2 (all terms positive: each TwoSum may take the larger sum first)
+PIC_HD dfl pr_one_plus_sqr(const dfl v[3]) {
+  dfl s(1.0f, 0.0f);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    k[d] = pr_mulf(h, eb[d]);
-    m[d] = pr_add(u[d], k[d]);
+  for (int d = 0; d < 3; ++d) s = pr_add_raw(s, pr_sqr(v[d]));
+  return pr_norm(s);
+}
+
+// The rotation of Boris, u+ = u- + (u- + u- x t) x 2 t/(1 + t^2), and of Higuera-Cary
+// (the same about t at its own gamma: w + w x t with (1 + t^2) w = u- + (u-.t) t + u- x t
+// is that rotation): du = u+ - u- of m = u-.  With t = c B, B exact in FP32, both cross
+// products run on B itself and only c and f = 2 c/(1 + t^2) are rounded; f is formed as
+// 2 (c - c t^2/(1 + t^2)), so that its error shrinks with t^2.  c^-2 is gamma^2/h^2 or
+// Higuera-Cary's gbar^2/h^2,
+//   gbar^2 = (sigma + root)/2, root^2 = sigma^2 + 4 (b^2 + (u-.b)^2), sigma = gamma^2 - b^2
+// (no cancellation in sigma: gbar <= gamma, so b^2 < gamma^2/16 below).  False outside
+// the pairs' range.
+template <bool HC>
+PIC_HD bool rotate_pair(const double m64[3], const float B[3], const PushConst& k, dfl du[3]) {
+  const uint32_t m0 = mag_word(m64[0]), m1 = mag_word(m64[1]), m2 = mag_word(m64[2]);
+  const uint32_t m01 = m0 > m1 ? m0 : m1, mm = m01 > m2 ? m01 : m2;
+  dfl m[3], v[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) m[d] = pr_split(m64[d]);
+  const dfl ih2(k.ih2_hi, k.ih2_lo), bb = pr_norm(pr_add_raw(
+      pr_add_raw(pr_mulff(B[0], B[0]), pr_mulff(B[1], B[1])), pr_mulff(B[2], B[2])));
+  dfl g2 = pr_norm(pr_mul(pr_one_plus_sqr(m), ih2));
+  // (also |t| and the products below within FP32: gamma^2/h^2 from 2^-40 to 2^80)
+  const bool inside = (mm == 0u || mm - mag_word_of(-64) < mag_word_of(40) - mag_word_of(-64)) &&
+                      g2.hi > 0x1p-40f && g2.hi < 0x1p80f;
+  if constexpr (HC) {
+    const dfl sg = pr_add(g2, pr_neg(bb));
+    const dfl w4 = pr_mul(ih2, pr_add(bb, pr_sqr(pr_dotf(m, B))));
+    const dfl q = pr_add(pr_sqr(sg), dfl(4.0f * w4.hi, 4.0f * w4.lo));
+    g2 = pr_add(sg, pr_norm(pr_mul(q, pr_rsqrt(q))));
+    g2 = dfl(0.5f * g2.hi, 0.5f * g2.lo);
   }
-  const dfl hig = pr_norm(pr_mul(h, pr_rsqrt(pr_one_plus_sqr(m))));
-#pragma unroll
-  for (int d = 0; d < 3; ++d) t[d] = pr_mulf(hig, eb[3 + d]);
-  dfl f = pr_rcp(pr_one_plus_sqr(t));
+  dfl c = pr_rsqrt(g2);
+  const dfl t2 = pr_norm(pr_mul(pr_norm(pr_sqr(c)), bb));
+  if (mag_sign(k.h)) c = pr_neg(c);
+  const dfl q = pr_norm(pr_mul(t2, pr_rcp(pr_add(dfl(1.0f, 0.0f), t2))));
+  dfl f = pr_add(c, pr_neg(pr_mul(c, q)));
   f = dfl(2.0f * f.hi, 2.0f * f.lo);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int a = (d + 1) % 3, b = (d + 2) % 3;
-    v[d] = pr_add(m[d], pr_det(m[a], t[b], m[b], t[a]));
-  }
+  for (int d = 0; d < 3; ++d) v[d] = pr_add(m[d], pr_mul(c, pr_crossf(m, B, (d + 1) % 3, (d + 2) % 3)));
 #pragma unroll
-  for (int d = 0; d < 3; ++d) t[d] = pr_mul(f, t[d]);
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int a = (d + 1) % 3, b = (d + 2) % 3;
-    du[d] = pr_add(pr_det(v[a], t[b], v[b], t[a]), dfl(2.0f * k[d].hi, 2.0f * k[d].lo));
-  }
+  for (int d = 0; d < 3; ++d) du[d] = pr_norm(pr_mul(f, pr_crossf(v, B, (d + 1) % 3, (d + 2) % 3)));
+  return inside && t2.hi < 0.0625f;   // (false for NaN)
 }
 
-// ---- Higuera-Cary: t = h B / gbar, w = (u- + (u-.t) t + u- x t)/(1 + t^2), u+ = w + w x t.
-// u+ - u- = 2 (w x t) (from w + t x w = u-, u+ = w + w x t), so du = 2 w x t + 2 h E.
-PIC_HD void hc_push_pair(dfl h, const float eb[6], const dfl u[3], dfl du[3]) {
-  dfl k[3], m[3], t[3], w[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    k[d] = pr_mulf(h, eb[d]);
-    m[d] = pr_add(u[d], k[d]);
-    t[d] = pr_norm(pr_mulf(h, eb[3 + d]));
-  }
-  // gbar^2 = (sigma + root)/2, root^2 = sigma^2 + 4 w4, sigma = gamma-^2 - b^2,
-  // w4 = b^2 + (u-.b)^2; for sigma < 0 the same root as 2 w4 / (root - sigma)
-  dfl b2 = pr_norm(pr_add_raw(pr_add_raw(pr_sqr(t[0]), pr_sqr(t[1])), pr_sqr(t[2])));
-  const dfl us = pr_norm(pr_add_raw(pr_add_raw(pr_mul(m[0], t[0]), pr_mul(m[1], t[1])), pr_mul(m[2], t[2])));
-  const dfl w4 = pr_add(b2, pr_sqr(us));
-  const dfl sigma = pr_add(pr_one_plus_sqr(m), pr_neg(b2));
-  const dfl q = pr_add(pr_sqr(sigma), dfl(4.0f * w4.hi, 4.0f * w4.lo));
-  const dfl root = pr_norm(pr_mul(q, pr_rsqrt(q)));
-  dfl g2;
-  if (sigma.hi >= 0.0f) {
-    g2 = pr_add(sigma, root);
-    g2 = dfl(0.5f * g2.hi, 0.5f * g2.lo);
-  } else {
-    g2 = pr_norm(pr_mul(dfl(2.0f * w4.hi, 2.0f * w4.lo), pr_rcp(pr_add(root, pr_neg(sigma)))));
-  }
-  const dfl ig = pr_rsqrt(g2);
-#pragma unroll
-  for (int d = 0; d < 3; ++d) t[d] = pr_norm(pr_mul(t[d], ig));
-  const dfl ut = pr_norm(pr_add_raw(pr_add_raw(pr_mul(m[0], t[0]), pr_mul(m[1], t[1])), pr_mul(m[2], t[2])));
-  const dfl s2 = pr_rcp(pr_one_plus_sqr(t));
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int a = (d + 1) % 3, b = (d + 2) % 3;
-    const dfl x = pr_add_raw(pr_mul(ut, t[d]), pr_det(m[a], t[b], m[b], t[a]));
-    w[d] = pr_norm(pr_mul(s2, pr_add(m[d], x)));
-  }
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int a = (d + 1) % 3, b = (d + 2) % 3;
-    const dfl x = pr_add(pr_det(w[a], t[b], w[b], t[a]), k[d]);
-    du[d] = dfl(2.0f * x.hi, 2.0f * x.lo);
-  }
-}
-
-// ---- analytic push (analytic_series.cuh) in s = (q/m) tau with the raw fields
-
-// sum of three exact products plus their low parts, normalised
+// sum of three pairs with exact high parts, normalised
 PIC_HD dfl pr_sum3(dfl a, dfl b, dfl c) {
   const dfl s = two_sum(a.hi, b.hi), r = two_sum(s.hi, c.hi);
   return fast_two_sum(r.hi, r.lo + (s.lo + ((a.lo + b.lo) + c.lo)));
 }
-PIC_HD void pr_apply(const float eb[6], const dfl V[4], dfl o[4]) {
+// s L V, L V = (E.v, V0 E + v x B)
+PIC_HD void pr_apply(const float eb[6], float s, const dfl V[4], dfl o[4]) {
   o[0] = pr_sum3(pr_mulf(V[1], eb[0]), pr_mulf(V[2], eb[1]), pr_mulf(V[3], eb[2]));
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const int a = (d + 1) % 3, b = (d + 2) % 3;
     o[d + 1] = pr_sum3(pr_mulf(V[0], eb[d]), pr_mulf(V[a + 1], eb[3 + b]), pr_mulf(V[b + 1], -eb[3 + a]));
   }
-}
-// D = (q/m) dt; du = u^{n+1/2} - u^{n-1/2}.  The root of F(s) = D is found in FP32
-// (as_start); one evaluation in pairs gives its residual delta, which then only
-// shifts the state to first order (|delta| <= 2^-21 |s|, so the second order is below
-// 2^-43 L s).  Returns false when the fields are beyond the series or the iteration
-// does not settle; the caller then takes the FP64 push.
-PIC_HD bool analytic_push_pair(dfl D, const float eb[6], const dfl u[3], dfl du[3]) {
-  dfl V[4][4];
-  const dfl x0 = pr_one_plus_sqr(u);
-  const dfl ig0 = pr_rsqrt(x0);
-  V[0][0] = pr_norm(pr_mul(x0, ig0));
 #pragma unroll
-  for (int d = 0; d < 3; ++d) V[0][d + 1] = u[d];
-  pr_apply(eb, V[0], V[1]);
-  pr_apply(eb, V[1], V[2]);
-  pr_apply(eb, V[2], V[3]);
+  for (int d = 0; d < 4; ++d) o[d] = pr_norm(pr_mulf(o[d], s));
+}
+
+// The analytic push (analytic_series.cuh) while L s is small, |s|^2 (E^2 + B^2) < 2^-6: U(s) =
+// U + s L U + R(s) in s = (q/m) tau with the raw fields; s L U, of size |L s| |U|, in
+// FP64 and R, of size |L s|^2 |U|/2, in pairs, so that R's rounding, 2^-48 of it, stays
+// below FP64's.  With b_k = s^k L^k U, A = S1 s^2, Q = S2 s^4 (|A| < 2^-6, Q < 2^-14) and
+// p_1 = 1, p_2 = A, p_3 = A^2 + Q, p_4 = A^3 + 2 A Q, s_a = sum_n p_n/(2n + a)!,
+//   R = s_0 b_2 + s_1 b_3 + Q s_2 U + Q s_3 b_1,
+//   F(s) = s [gamma + b_1/2 + s_1 b_2 + s_2 b_3 + Q s_3 gamma + Q s_4 b_1] (time components)
+// is q/m times the lab time.  An FP32 Newton gives s to about 2^-22, the FP64 residual
+// F(s) - (q/m) dt the rest, delta, which moves s in the FP64 term and R to second order.
+// False outside, with u unchanged.
+PIC_HD bool analytic_push_weak(double D, const float eb[6], double u[3]) {
+  const uint32_t m0 = mag_word(u[0]), m1 = mag_word(u[1]), m2 = mag_word(u[2]);
+  const uint32_t m01 = m0 > m1 ? m0 : m1, mm = m01 > m2 ? m01 : m2;
+  bool inside = mm < mag_word_of(40);
+  const double x0 = 1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  const double ig0 = rsqrt_nr(x0), g0 = x0 * ig0;
+  double E[6], LU[4];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) E[c] = widen(eb[c]);
+  LU[0] = E[0] * u[0] + E[1] * u[1] + E[2] * u[2];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const int a = (d + 1) % 3, b = (d + 2) % 3;
+    LU[d + 1] = fma(g0, E[d], fma(u[a], E[3 + b], -(u[b] * E[3 + a])));
+  }
+  const float Df = narrow_sat(D), ig = narrow_sat(ig0);
   const dfl ee = pr_sum3(pr_mulff(eb[0], eb[0]), pr_mulff(eb[1], eb[1]), pr_mulff(eb[2], eb[2]));
   const dfl bb = pr_sum3(pr_mulff(eb[3], eb[3]), pr_mulff(eb[4], eb[4]), pr_mulff(eb[5], eb[5]));
   const dfl dot = pr_sum3(pr_mulff(eb[0], eb[3]), pr_mulff(eb[1], eb[4]), pr_mulff(eb[2], eb[5]));
-  const dfl S1 = pr_add(ee, pr_neg(bb)), S2 = pr_norm(pr_sqr(dot));
-  dfl s = pr_norm(pr_mul(D, ig0));
+  const float sa = Df * ig;
+  inside = inside && sa * sa * (ee.hi + bb.hi) < 0.015625f && fabsf(Df) > 0x1p-20f && fabsf(Df) < 0x1p20f;
+  if (!inside) return false;                        // (also NaN)
+  dfl V0[4], b1[4], b2[4], b3[4];
+  V0[0] = pr_split(g0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) V0[d + 1] = pr_split(u[d]);
+  dfl W1[4];
+#pragma unroll
+  for (int d = 0; d < 4; ++d) W1[d] = pr_split(LU[d]);
+  // s in FP32: Newton on s (1 + s (p/2 + s (r/6 + s t/24))) = D/gamma, L^k U in FP32
+  float s = sa;
   {
-    const float Vf[4] = {V[0][0].hi, V[1][0].hi, V[2][0].hi, V[3][0].hi};
-    const float s0 = s.hi;
-    const float d = as_start(Vf, S1.hi, S2.hi, D.hi, s0) - s0;
-    if (d != 0.0f) s = pr_add(s, dfl(d, 0.0f));
-  }
-#pragma unroll 1
-  for (int it = 0; it < 6; ++it) {
-    const dfl z = pr_norm(pr_sqr(s));
-    const dfl A = pr_norm(pr_mul(S1, z)), Q = pr_norm(pr_mul(S2, pr_norm(pr_sqr(z))));
-    if (!as_series_ok(A.hi, Q.hi)) return false;
-    const int K = as_terms(PIC_AS.t48, as_root_max(A.hi, Q.hi));
-    dfl e1(0.0f, 0.0f), o1(0.0f, 0.0f), e0(PIC_AS.h2[K - 1], PIC_AS.l2[K - 1]), o0(PIC_AS.h3[K - 1], PIC_AS.l3[K - 1]);
-#pragma unroll 1
-    for (int n = K - 2; n >= 0; --n) {
-      const dfl en = pr_sum3(dfl(PIC_AS.h2[n], PIC_AS.l2[n]), pr_mul(A, e0), pr_mul(Q, e1));
-      const dfl on = pr_sum3(dfl(PIC_AS.h3[n], PIC_AS.l3[n]), pr_mul(A, o0), pr_mul(Q, o1));
-      e1 = e0;
-      o1 = o0;
-      e0 = en;
-      o0 = on;
+    float w[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int a = (d + 1) % 3, b = (d + 2) % 3;
+      w[d] = fmaf(W1[0].hi, eb[d], fmaf(W1[a + 1].hi, eb[3 + b], -(W1[b + 1].hi * eb[3 + a])));
     }
-    const dfl q2 = pr_norm(pr_mul(Q, e1));
-    const dfl c1 = pr_add(s, pr_mul(s, pr_norm(pr_mul(Q, o1))));
-    const dfl c2 = pr_norm(pr_mul(z, e0)), c3 = pr_norm(pr_mul(pr_norm(pr_mul(z, s)), o0));
-    const dfl d1 = pr_norm(pr_mul(z, pr_add(e0, pr_neg(pr_mul(A, e1)))));
-    const dfl d3 = pr_norm(pr_mul(pr_norm(pr_sqr(z)), e1));
-    // residual F(s) - D and gamma(s) (FP32: it only scales the residual)
-    const dfl F = pr_add(pr_add_raw(pr_mul(c1, V[0][0]), pr_mul(d1, V[1][0])),
-                         pr_add_raw(pr_mul(c3, V[2][0]), pr_mul(d3, V[3][0])));
-    const float gam = V[0][0].hi + fmaf(c3.hi, V[3][0].hi, fmaf(c2.hi, V[2][0].hi, fmaf(c1.hi, V[1][0].hi, q2.hi * V[0][0].hi)));
-    const dfl r = pr_add_raw(F, pr_neg(D));
-    const float delta = -(r.hi + r.lo) / gam;
-    if (!(fabsf(delta) < fabsf(s.hi))) return false;   // also NaN
-    if (fabsf(delta) <= 4.76837158203125e-7f * fabsf(s.hi)) {
-      // u(s) - u(0), then delta du/ds = delta (gamma E + u(s) x B) in FP32
-      float un[3];
+    const float p = 0.5f * (W1[0].hi * ig);
+    const float r = 0.16666667f * (fmaf(eb[0], W1[1].hi, fmaf(eb[1], W1[2].hi, eb[2] * W1[3].hi)) * ig);
+    const float t = 0.041666668f * (fmaf(eb[0], w[0], fmaf(eb[1], w[1], eb[2] * w[2])) * ig);
 #pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        du[d] = pr_add(pr_add_raw(pr_mul(q2, u[d]), pr_mul(c1, V[1][d + 1])),
-                       pr_add_raw(pr_mul(c2, V[2][d + 1]), pr_mul(c3, V[3][d + 1])));
-        un[d] = u[d].hi + du[d].hi;
-      }
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const int a = (d + 1) % 3, b = (d + 2) % 3;
-        const float g = fmaf(gam, eb[d], fmaf(un[a], eb[3 + b], -(un[b] * eb[3 + a])));
-        du[d] = pr_add(du[d], dfl(delta * g, 0.0f));
-      }
-      return true;
-    }
-    s = pr_add(s, dfl(delta, 0.0f));
-  }
-  return false;
-}
-
-// ---- one particle: u (FP64, in and out) and the pair dx[d] of its move over dt
-// along the first ndim axes, 1/gamma and u^{n+1/2} in FP32.  Returns false when the
-// analytic push did not converge (u unchanged).
-struct PairMove {
-  dfl dx[3];
-  float dtig, ig, u[3];   // dt/gamma, 1/gamma, u^{n+1/2}
-};
-
-PIC_HDI bool push_wide(double qm, double dt, int kind, const float eb[6], double u[3]);
-
-// max |v_d| below 2^e (e > 0), false for NaN; on the integer pipe
-PIC_HD bool pr_below(const double v[3], int e) {
-  const uint32_t m = 0x7fffffffu;
-  const uint32_t a = (uint32_t)(f64_bits(v[0]) >> 32) & m, b = (uint32_t)(f64_bits(v[1]) >> 32) & m,
-                 c = (uint32_t)(f64_bits(v[2]) >> 32) & m;
-  const uint32_t ab = a > b ? a : b;
-  return (ab > c ? ab : c) < (uint32_t)(1023 + e) << 20;
-}
-
-template <int PUSH, int NDIM>
-PIC_HD bool push_pair(double qm, double dt, int pusher, const float eb[6], double u[3], PairMove& mv) {
-  // The pairs hold |u| and |q/m dt E|, |q/m dt B| below 2^28 (gamma^4 within FP32 in the
-  // Higuera-Cary root); anything else, infinities and NaN among it, takes the FP64
-  // push, which either moves the particle or gives a non-finite dt/gamma.
-  const int kind = PUSH < 0 ? pusher : PUSH;
-  const float k = fabsf(narrow_sat(qm * dt));
-  float em = 0.0f;
-  bool inside = pr_below(u, 28);
-#pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    em = fmaxf(em, fabsf(eb[c]));
-    inside = inside && eb[c] == eb[c];
-  }
-  inside = inside && k * em < 0x1p28f;
-  double un[3] = {u[0], u[1], u[2]};
-  if (inside) {
-    dfl U[3], du[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) U[d] = pr_split(u[d]);
-    if (kind == PIC_ANALYTIC) {
-      inside = analytic_push_pair(pr_split(qm * dt), eb, U, du);
-    } else if (kind == PIC_HC) {
-      hc_push_pair(pr_split(0.5 * qm * dt), eb, U, du);
-    } else {
-      boris_push_pair(pr_split(0.5 * qm * dt), eb, U, du);
-    }
-#pragma unroll
-    for (int d = 0; d < 3; ++d) un[d] += pr_join(du[d]);
-    inside = inside && pr_below(un, 60);
-    if (inside) {
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        u[d] = un[d];
-        U[d] = pr_add(U[d], du[d]);
-      }
-      const dfl ig = pr_rsqrt(pr_one_plus_sqr(U));
-      const dfl dtig = pr_norm(pr_mul(pr_split(dt), ig));
-#pragma unroll
-      for (int d = 0; d < NDIM; ++d) mv.dx[d] = pr_mul(dtig, U[d]);
-      mv.dtig = dtig.hi;
-      mv.ig = ig.hi;
-#pragma unroll
-      for (int d = 0; d < 3; ++d) mv.u[d] = U[d].hi;
-      return true;
+    for (int it = 0; it < 3; ++it) {
+      const float F = fmaf(s * s, fmaf(s, fmaf(s, t, r), p), s - sa);
+      const float G = s * fmaf(s, fmaf(s, 4.0f * t, 3.0f * r), 2.0f * p);   // dF/ds - 1, small
+      s = fmaf(-F, fmaf(G, G, 1.0f - G), s);
     }
   }
-  if (!push_wide(qm, dt, kind, eb, u)) return false;
-  const double ig = rsqrt_nr<1>(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-  const double dtig = dt * ig;
-  // (a non-finite dt/gamma must reach the caller's check as such)
-  mv.dtig = isfinite(dtig) ? narrow_signed(dtig) : NAN;
-  mv.ig = narrow_signed(ig);
+#pragma unroll
+  for (int d = 0; d < 4; ++d) b1[d] = pr_norm(pr_mulf(W1[d], s));
+  pr_apply(eb, s, b1, b2);
+  pr_apply(eb, s, b2, b3);
+  const dfl z = pr_mulff(s, s);
+  const dfl A = pr_norm(pr_mul(pr_add(ee, pr_neg(bb)), z)), dz = pr_norm(pr_mul(dot, z)), Q = pr_norm(pr_sqr(dz));
+  const float p3 = fmaf(A.hi, A.hi, Q.hi), p4 = A.hi * fmaf(A.hi, A.hi, 2.0f * Q.hi);
+  // 1/3!, 1/4!, 1/5! as pairs
+  const dfl i6(PIC_AS.h3[0], PIC_AS.l3[0]), i24(PIC_AS.h2[1], PIC_AS.l2[1]), i120(PIC_AS.h3[1], PIC_AS.l3[1]);
+  const dfl s0 = pr_sum3(dfl(0.5f, 0.0f), pr_mul(A, i24), dfl(fmaf(p4, PIC_AS.h2[3], p3 * PIC_AS.h2[2]), 0.0f));
+  const dfl s1 = pr_sum3(i6, pr_mul(A, i120), dfl(fmaf(p4, PIC_AS.h3[3], p3 * PIC_AS.h3[2]), 0.0f));
+  const dfl s2 = pr_add(i24, dfl(fmaf(p3, PIC_AS.h2[3], A.hi * PIC_AS.h2[2]), 0.0f));
+  const dfl q3 = pr_norm(pr_mul(Q, pr_add(i120, dfl(A.hi * PIC_AS.h3[2], 0.0f))));
+  const float q4 = Q.hi * fmaf(A.hi, PIC_AS.h2[3], PIC_AS.h2[2]);
+  const dfl q2 = pr_norm(pr_mul(Q, s2));
+  dfl Rf = pr_add(pr_add_raw(pr_mul(s1, b2[0]), pr_mul(s2, b3[0])), pr_add_raw(pr_mul(q3, V0[0]), dfl(q4 * b1[0].hi, 0.0f)));
+  const double s64 = widen(s);
+  const double r = fma(s64, fma(0.5 * s64, LU[0], g0) + pr_join(Rf), -D);
+  const float Rg = fmaf(s0.hi, b2[0].hi, fmaf(s1.hi, b3[0].hi, fmaf(q2.hi, V0[0].hi, q3.hi * b1[0].hi)));
+  const double gam = fma(s64, LU[0], g0) + widen(Rg);
+  const double rg = rcp_nr<1>(gam), d1 = -r * rg;
+  const float d1f = narrow_signed(d1), e = d1f * seed_rcp(s);   // delta, delta/s
+  // second order of Newton: -(gamma'/2 gamma) delta^2
+  const float d2 = -0.5f * narrow_signed(rg) * (b1[0].hi + fmaf(0.5f, b3[0].hi, b2[0].hi)) * (e * d1f);
+  if (!(fabsf(e) <= 0x1p-20f)) return false;         // not settled, NaN
+  const double sn = s64 + (d1 + widen(d2));
+  // R(s + delta) = R + delta L (s L U + R) + (delta^2/2) L^2 U
+  dfl R[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    R[d] = pr_add(pr_add_raw(pr_mul(s0, b2[d + 1]), pr_mul(s1, b3[d + 1])),
+                  pr_add_raw(pr_mul(q2, V0[d + 1]), pr_mul(q3, b1[d + 1])));
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    if (d < NDIM) mv.dx[d] = pr_split(dtig * u[d]);
-    mv.u[d] = narrow_signed(u[d]);
+    const int a = (d + 1) % 3, b = (d + 2) % 3;
+    const float T = s * fmaf(Rg, eb[d], fmaf(R[a].hi, eb[3 + b], -(R[b].hi * eb[3 + a])));
+    const float dR = e * (fmaf(0.5f * e, b2[d + 1].hi, b2[d + 1].hi) + T);
+    u[d] = fma(sn, LU[d + 1], u[d] + pr_join(pr_add(R[d], dfl(dR, 0.0f))));
   }
   return true;
 }
 
-// the FP64 push of a particle in FP32 fields (out of line)
+// The FP64 push next to FP32 fields, out of line for the rare particles outside the
+// pairs' range (arguments and result by value: the caller's stay in registers).  ok:
+// false when the analytic push did not converge.
+struct PushState {
+  double u[3];
+  float eb[6];
+  bool ok;
+};
+template <int KIND>
 #ifdef __CUDA_ARCH__
 __noinline__
 #endif
-PIC_HDI bool push_wide(double qm, double dt, int kind, const float eb[6], double u[3]) {
+PIC_HDI PushState push_wide(double qm, double dt, PushState s) {
   double e[6];
-  for (int c = 0; c < 6; ++c) e[c] = (double)eb[c];
-  double v[3] = {u[0], u[1], u[2]};
-  if (kind == PIC_ANALYTIC) {
-    if (analytic_push_series(qm, dt, e, v) < 0) return false;
-  } else if (kind == PIC_HC) {
-    hc_push<1>(qm, dt, e, v);
+  for (int c = 0; c < 6; ++c) e[c] = widen(s.eb[c]);
+  if constexpr (KIND == PIC_ANALYTIC) s.ok = analytic_push_series(qm, dt, e, s.u) > 0;
+  else if constexpr (KIND == PIC_HC) hc_push<1>(qm, dt, e, s.u);
+  else boris_push<1>(qm, dt, e, s.u);
+  return s;
+}
+
+// ---- one particle: u (in and out), dt/gamma, 1/gamma of u^{n+1/2}, and its move
+// dx[d] = (dt/gamma) u_d, which takes one fused multiply-add onto the position.
+// Returns false when the analytic push did not converge (u unchanged).
+struct Move {
+  double v, u;
+};
+PIC_HD double pr_join(Move m) { return m.v * m.u; }
+struct PairMove {
+  Move dx[3];
+  double dtig, ig;
+};
+
+template <int KIND>
+PIC_HD bool push_kind(double qm, double dt, const PushConst& k, const float eb[6], double u[3]) {
+  if constexpr (KIND == PIC_ANALYTIC) {
+    if (analytic_push_weak(2.0 * k.h, eb, u)) return true;
   } else {
-    boris_push<1>(qm, dt, e, v);
+    double e[3], m[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      e[d] = widen(eb[d]);
+      m[d] = fma(k.h, e[d], u[d]);
+    }
+    dfl du[3];
+    if (rotate_pair<KIND == PIC_HC>(m, eb + 3, k, du)) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) u[d] = fma(k.h, e[d], m[d] + pr_join(du[d]));
+      return true;
+    }
   }
-  for (int d = 0; d < 3; ++d) u[d] = v[d];
+  const PushState w = push_wide<KIND>(
+      qm, dt, PushState{{u[0], u[1], u[2]}, {eb[0], eb[1], eb[2], eb[3], eb[4], eb[5]}, true});
+  if (!w.ok) return false;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) u[d] = w.u[d];
   return true;
+}
+
+template <int PUSH, int NDIM>
+PIC_HD bool push_pair(double qm, double dt, const PushConst& k, int pusher, const float eb[6],
+                      double u[3], PairMove& mv) {
+  const int kind = PUSH < 0 ? pusher : PUSH;
+  bool ok;
+  if (kind == PIC_ANALYTIC) ok = push_kind<PIC_ANALYTIC>(qm, dt, k, eb, u);
+  else if (kind == PIC_HC) ok = push_kind<PIC_HC>(qm, dt, k, eb, u);
+  else ok = push_kind<PIC_BORIS>(qm, dt, k, eb, u);
+  if (!ok) return false;
+  mv.ig = rsqrt_nr<1>(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+  mv.dtig = dt * mv.ig;
+#pragma unroll
+  for (int d = 0; d < NDIM; ++d) mv.dx[d] = Move{mv.dtig, u[d]};
+  return true;
+}
+template <int PUSH, int NDIM>
+PIC_HD bool push_pair(double qm, double dt, int pusher, const float eb[6], double u[3], PairMove& mv) {
+  return push_pair<PUSH, NDIM>(qm, dt, push_const(qm, dt), pusher, eb, u, mv);
 }
 
 }  // namespace pic

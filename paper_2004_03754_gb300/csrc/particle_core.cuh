@@ -1,7 +1,8 @@
 // particle_core.cuh -- per-particle device code shared by the tiled particle
 // kernel, the straggler kernel and the persistent ensemble kernel:
 //   gather (App. A, quadratic B-spline at each component's staggered node)
-//   -> push (Boris or analytic, FP64) -> x^{n+1} = x^n + dt u/gamma (FP64)
+//   -> push (FP64; next to FP32 fields with parts in FP32 pairs, pair_push.cuh; the
+//      ensembles' in FP64 throughout) -> x^{n+1} = x^n + dt u/gamma (FP64)
 //   -> Esirkepov deposit (Sec. 3.3).
 // Field access goes through "views" (shared-memory window or global memory with
 // periodic wrap) and current accumulation through "accumulators".
@@ -750,9 +751,8 @@ PIC_HD void advance_particle(const VE* ve, const VB* vb, const ACC* acc,
                                                  const PartPtrs& p, int64_t q, const int* li,
                                                  const T* f, const int* gcell, const GridArgs& g,
                                                  const PartArgs& a, unsigned* err) {
-  // FP32 fields: the push in FP32 pairs, its changes of u and x added in FP64
-  // (pair_push.cuh).  FP64 and compensated fields: the FP64 push, reciprocals by
-  // two Newton steps.
+  // FP32 fields: FP64 with the rotation in FP32 pairs (pair_push.cuh), reciprocals by
+  // one Newton step; FP64 and compensated fields: the FP64 push, two Newton steps.
   constexpr bool F32 = std::is_same<T, float>::value, PAIR = F32 && !TEST;
   constexpr int NR = F32 ? 1 : 2;
   using D = typename DepositOf<T>::type;
@@ -770,18 +770,17 @@ PIC_HD void advance_particle(const VE* ve, const VB* vb, const ACC* acc,
   double u[3] = {p.u[0][q], p.u[1][q], p.u[2][q]};
   const double um[3] = {u[0], u[1], u[2]};
   double dx[3];   // the move, FP64 (FP64 and compensated fields)
-  PairMove mv;    // the move in FP32 pairs (FP32 fields)
-  double ig = 0.0, dtig = 0.0;
+  double ig, dtig;   // 1/gamma, dt/gamma
   T delta[3];     // the move in cells, in the field precision (shape weights)
-  bool moved_ok = true, finite;
+  bool moved_ok = true;
   if constexpr (PAIR) {
-    if (!push_pair<PUSH, NDIM>(a.qm, g.dt, a.pusher, eb, u, mv)) {
+    PairMove mv;
+    if (!push_pair<PUSH, NDIM>(a.qm, g.dt, a.push, a.pusher, eb, u, mv)) {
       latch(err, ERRBIT_ANALYTIC);
       return;
     }
-    finite = isfinite(mv.dtig);
-#pragma unroll
-    for (int d = 0; d < NDIM; ++d) delta[d] = mv.dtig * mv.u[d] * to_prec<float>(g.inv_dx[d]);
+    ig = mv.ig;
+    dtig = mv.dtig;
   } else {
     if (PUSH == PIC_ANALYTIC || (PUSH < 0 && a.pusher == PIC_ANALYTIC)) {
       const int it = TEST ? analytic_push(a.qm, g.dt, eb, u) : analytic_push_series(a.qm, g.dt, eb, u);
@@ -796,31 +795,31 @@ PIC_HD void advance_particle(const VE* ve, const VB* vb, const ACC* acc,
     }
     ig = rsqrt_nr<NR>(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
     dtig = g.dt * ig;
-    finite = isfinite(dtig);
-#pragma unroll
-    for (int d = 0; d < NDIM; ++d) {
-      if constexpr (F32) {
-        delta[d] = to_prec<float>(dtig) * to_prec<float>(u[d]) * to_prec<float>(g.inv_dx[d]);
-      } else {
-        dx[d] = dtig * u[d];
-        if constexpr (is_dfl<T>::value) delta[d] = T(dx[d] * g.inv_dx[d]);
-        else delta[d] = dx[d] * g.inv_dx[d];
-      }
-    }
   }
   if constexpr (GAIN) {
     const double gm2 = 1.0 + um[0] * um[0] + um[1] * um[1] + um[2] * um[2];
     const double gp2 = 1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    // gamma^{n-1/2} + gamma^{n+1/2}
-    const double gsum = gm2 * rsqrt_nr<NR>(gm2) + gp2 * rsqrt_nr<NR>(gp2);
+    const double gsum = gm2 * rsqrt_nr<NR>(gm2) + gp2 * ig;   // gamma^{n-1/2} + gamma^{n+1/2}
     const double w = a.qm * g.dt * rcp_nr<NR>(gsum);
     p.wl[q] += w * (double)eb[0] * (um[0] + u[0]);
     p.wd[q] += w * ((double)eb[1] * (um[1] + u[1]) + (double)eb[2] * (um[2] + u[2]));
   }
+  // FP32 fields: the move in cells is formed from the narrowed factors, and the FP64
+  // position takes the move as one fused multiply-add per axis.  FP64 and compensated
+  // fields: the FP64 move dx, its cells and the position from it.
 #pragma unroll
-  for (int d = 0; d < NDIM; ++d) moved_ok = moved_ok && below_one(delta[d]);   // false for NaN
-  if (!moved_ok) {
-    latch(err, finite ? ERRBIT_MOVE : ERRBIT_NONFINITE);
+  for (int d = 0; d < NDIM; ++d) {
+    if constexpr (F32) {
+      delta[d] = to_prec<float>(dtig) * to_prec<float>(u[d]) * to_prec<float>(g.inv_dx[d]);
+    } else {
+      dx[d] = dtig * u[d];
+      if constexpr (is_dfl<T>::value) delta[d] = T(dx[d] * g.inv_dx[d]);
+      else delta[d] = dx[d] * g.inv_dx[d];
+    }
+    moved_ok = moved_ok && below_one(delta[d]);   // false for NaN
+  }
+  if (!moved_ok || !isfinite(dtig)) {
+    latch(err, isfinite(dtig) ? ERRBIT_MOVE : ERRBIT_NONFINITE);
     return;
   }
   const double w = p.w[q];
@@ -835,8 +834,7 @@ PIC_HD void advance_particle(const VE* ve, const VB* vb, const ACC* acc,
     }
     // w v3 = w u3 / gamma; in FP32 as the product of the narrowed factors
     D v3;
-    if constexpr (PAIR) v3 = mv.u[2] * mv.ig;
-    else if constexpr (std::is_same<D, float>::value) v3 = to_prec<D>(u[2]) * to_prec<D>(ig);
+    if constexpr (std::is_same<D, float>::value) v3 = to_prec<D>(u[2]) * to_prec<D>(ig);
     else v3 = to_prec<D>(u[2] * ig);
     if constexpr (std::is_same<ACC, FixAcc64>::value) deposit_fixed<NDIM>(acc, li, fd, dd, cf, wt * v3);
     else deposit<D, NDIM>(acc, li, fd, dd, cf, wt * v3);
@@ -847,8 +845,7 @@ PIC_HD void advance_particle(const VE* ve, const VB* vb, const ACC* acc,
 #pragma unroll
   for (int d = 0; d < NDIM; ++d) {
     double x;
-    if constexpr (PAIR) x = p.x[d][q] + pr_join(mv.dx[d]);
-    else if constexpr (F32) x = fma(dtig, u[d], p.x[d][q]);
+    if constexpr (F32) x = fma(dtig, u[d], p.x[d][q]);
     else x = p.x[d][q] + dx[d];
     const int land = gcell[d] + (int)floorf(rough(f[d]) + rough(delta[d]));
     if (land <= 0 || land >= g.n[d] - 1) {

@@ -8,7 +8,8 @@
 // over the grid.  One CTA owns one tile: it stages E^n and B^n of the tile plus
 // a guard in shared memory and runs every particle of the bin through
 //   gather (App. A, quadratic B-spline at each component's staggered node)
-//   -> push (Boris, Higuera-Cary or analytic, FP64)
+//   -> push (Boris, Higuera-Cary or analytic, FP64; next to FP32 fields the parts of
+//      it that lose nothing by it in FP32 pairs, pair_push.cuh)
 //   -> x^{n+1} = x^n + dt u/gamma (FP64)
 //   -> Esirkepov deposit (Sec. 3.3) into a shared-memory current window (int32
 //      fixed point),
@@ -70,6 +71,20 @@ __device__ __forceinline__ void red_add4(float* p, const float* v) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
                "f"(v[3])
                : "memory");
+}
+
+// cell of a coordinate in cells and the fraction in the field precision (exact, rounded
+// once; no FP64 conversion)
+template <typename T>
+__device__ __forceinline__ int cell_split(double c, T& f) {
+  if constexpr (std::is_same<T, float>::value) {
+    return floor_split(c, f);
+  } else {
+    double frac;
+    const int k = floor_split(c, frac);
+    f = to_prec<T>(frac);
+    return k;
+  }
 }
 
 // threads 0 .. NDIM+3 ask L2 for one particle array each over [c0, c1) (bulk
@@ -271,10 +286,7 @@ __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::c
     bool inside = true;
 #pragma unroll
     for (int d = 0; d < NDIM; ++d) {
-      const double c = p.x[d][q] * g.inv_dx[d];
-      double frac;
-      gc[d] = floor_split(c, frac);             // exact floor and fraction, no FP64 conversion
-      fr[d] = to_prec<T>(frac);
+      gc[d] = cell_split(p.x[d][q] * g.inv_dx[d], fr[d]);
       int l = gc[d] - wlo[d];
       if (l < ulo[d]) l += g.n[d];
       else if (l >= uhi[d]) l -= g.n[d];
@@ -382,10 +394,7 @@ __global__ void straggler_kernel(FieldPtrs<T> f, BbarPtrs<T> bg, PartPtrs p, Gri
     T fr[3];
 #pragma unroll
     for (int d = 0; d < NDIM; ++d) {
-      const double c = p.x[d][q] * g.inv_dx[d];
-      double frac;
-      li[d] = floor_split(c, frac);
-      fr[d] = to_prec<T>(frac);
+      li[d] = cell_split(p.x[d][q] * g.inv_dx[d], fr[d]);
     }
     advance_particle<T, NDIM, -1, GAIN>(ve, vb, acc, p, q, li, fr, li, g, a, bins.err);
   }
@@ -408,9 +417,7 @@ __global__ void __launch_bounds__(128) sparse_kernel(FieldPtrs<T> f, BbarPtrs<T>
     T fr[3];
 #pragma unroll
     for (int d = 0; d < NDIM; ++d) {
-      double frac;
-      gc[d] = floor_split(p.x[d][q] * g.inv_dx[d], frac);
-      fr[d] = to_prec<T>(frac);
+      gc[d] = cell_split(p.x[d][q] * g.inv_dx[d], fr[d]);
     }
     const int o3 = NDIM == 3 ? gc[2] - 1 : 0;
     for (int m = lane; m < NODES; m += 32) {
