@@ -157,6 +157,7 @@ pic_status build_correction(pic_ctx* c) {
 void free_shares(pic_ctx* c) {
   pic::TileShares& h = c->bins.share;
   cudaFree(h.counts);
+  cudaFree(h.line);
   cudaFree(h.list);
   cudaFree(h.slot);
   cudaFree(h.scratch);
@@ -177,7 +178,8 @@ pic_status alloc_shares(pic_ctx* c, int64_t n) {
     h.words = 4 + (particle_window_ints(c->grid.ndim, c->grid.precision == PIC_FP64, c->tsize,
                                         c->ptile) + 3) / 4 * 4;
     const size_t bytes = sizeof(int) * (size_t)h.words * most;
-    if (cudaMalloc(&h.counts, 2 * sizeof(int)) != cudaSuccess ||
+    if (cudaMalloc(&h.counts, 3 * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&h.line, sizeof(int64_t)) != cudaSuccess ||
         cudaMalloc(&h.list, sizeof(pic::TileShare) * most) != cudaSuccess ||
         cudaMalloc(&h.slot, sizeof(int) * c->ptile.ntiles) != cudaSuccess ||
         cudaMalloc(&h.scratch, bytes) != cudaSuccess) {
@@ -186,6 +188,7 @@ pic_status alloc_shares(pic_ctx* c, int64_t n) {
       return PIC_OK;
     }
     CK(c, cudaMemsetAsync(h.scratch, 0, bytes, c->stream));
+    CK(c, cudaMemsetAsync(h.counts, 0, 3 * sizeof(int), c->stream));
     h.ntiles = c->ptile.ntiles;
     h.cap = most;
   }

@@ -178,26 +178,41 @@ inline PartArgs part_args(double qm, double dt, int pusher, int64_t np) {
 // warps, two per SM, end before a tile has staged its window.
 __host__ __device__ inline bool particles_sparse(bool f64, int64_t np) { return f64 && np <= 256; }
 
-// Crowded tiles: a tile of more than `chunk` particles is shared by several CTAs (its
-// time would otherwise bound the whole step: an electron sheet in front of a strong
-// pulse put 12 times the mean into one tile).  Each share runs in a current window of
-// its own, on the scales of the whole tile; the windows' integers are added up in
-// `scratch` and the last CTA to arrive flushes the sum, so the current does not depend
-// on the split.  The list is made with the tile counts of each re-binning.  The line
-// is a quarter of what an SM gets of all particles: four tiles of that size are
+// Crowded tiles: a tile of more than `line` particles is shared by several CTAs of up to
+// `chunk` each (its time would otherwise bound the whole step: an electron sheet in front
+// of a strong pulse put 12 times the mean into one tile).  Each share runs in a current
+// window of its own, on the scales of the whole tile; the windows' integers are added up
+// in `scratch` and the last CTA to arrive flushes the sum, so the current does not depend
+// on the split.  The list is made with the tile counts of each re-binning.
+// A share is a quarter of what an SM gets of all particles: four tiles of that size are
 // resident on an SM at least in part, so a smaller one does not stand out; and never
 // under 1024 particles, where staging the windows again costs what the split gives.
 // 2D compensated, 1.5 M electrons behind a pulse of a0 = 100, particle kernel per
 // step: largest tile 3.2 k particles 0.75 -> 0.79 ms, 9.4 k 1.18 -> 0.89, 12 k
 // 1.39 -> 0.94; with no crowded tile 1.58 -> 1.56 (29.4 M electrons, mixed) and
 // 2.16 -> 2.16 ms (6.3 M, FP64).
+// The line (share_line) is a share, but at least half more than the mean of the occupied
+// tiles: where few tiles hold a uniform plasma, every one of them is larger than a share
+// and splitting them all only adds windows (1024x256 in 512 tiles, 4 electrons per cell,
+// eight steps: mixed 1.49 -> 1.05 ms, compensated 3.28 -> 2.61, FP64 5.19 -> 4.62 with the
+// tiles whole; 48^3, 8 per cell, four steps 1.66 -> 1.33).  Past what an SM gets of all
+// particles a tile is always split: there are fewer tiles than SMs, or one is a sheet
+// (256x128 in 64 tiles, 8 per cell, 0.53 ms split and 0.61 whole).
+__host__ __device__ inline int64_t share_line(int64_t particles, int64_t occupied, int64_t chunk) {
+  const int64_t half_more = occupied > 0 ? (3 * particles + 2 * occupied - 1) / (2 * occupied) : 0;
+  const int64_t sm = (particles + 151) / 152;
+  const int64_t line = half_more < sm ? half_more : sm;
+  return line > chunk ? line : chunk;
+}
 struct TileShare {
   int tile, part, slot;
 };
 struct TileShares {
   int64_t chunk;      // particles per share; 0: no list
   int64_t ntiles;
-  int* counts;        // [0] shares beyond the first of their tiles, [1] crowded tiles
+  int* counts;        // [0] shares beyond the first of their tiles, [1] crowded tiles,
+                      // [2] occupied tiles while they are counted
+  int64_t* line;      // most particles of a tile that is not shared
   TileShare* list;    // the former
   int* slot;          // ntiles: index of a crowded tile
   int* scratch;       // per crowded tile: arrival count (16 bytes), then the window's integers

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::c
   // (in shared memory: read again after the particle loop, no registers held across it)
   __shared__ int s_parts, s_slot;
   if (threadIdx.x == 0) s_parts = 1;
-  if (bins.share.chunk > 0 && tend - tbeg > bins.share.chunk) {
+  if (bins.share.chunk > 0 && tend - tbeg > *bins.share.line) {
     const int parts = (int)((tend - tbeg + bins.share.chunk - 1) / bins.share.chunk);
     const int64_t per = (tend - tbeg + parts - 1) / parts;
     pbeg = min(tend, tbeg + part * per);

@@ -58,9 +58,17 @@ __global__ void __launch_bounds__(kScanT) bin_chunk_sum_kernel(BinBufs b, int64_
   __shared__ int64_t ws[kScanT / 32];
   const int64_t base = (int64_t)blockIdx.x * kScanChunk + threadIdx.x * kScanPer;
   int64_t s = 0;
+  int occupied = 0;
 #pragma unroll
   for (int k = 0; k < kScanPer; ++k)
-    if (base + k < n) s += b.count[base + k];
+    if (base + k < n) {
+      s += b.count[base + k];
+      occupied += b.count[base + k] != 0 && base + k < b.share.ntiles;
+    }
+  if (b.share.chunk > 0) {
+    occupied = __reduce_add_sync(0xffffffffu, occupied);
+    if ((threadIdx.x & 31) == 0 && occupied != 0) atomicAdd(&b.share.counts[2], occupied);
+  }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
   __syncthreads();
@@ -97,7 +105,7 @@ __global__ void __launch_bounds__(kScanT) bin_chunk_out_kernel(BinBufs b, int64_
     if (base + k < n) b.start[base + k] = run;
     run += v[k];
     // shares of a crowded tile beyond its first
-    if (b.share.chunk > 0 && v[k] > b.share.chunk && base + k < b.share.ntiles) {
+    if (b.share.chunk > 0 && v[k] > *b.share.line && base + k < b.share.ntiles) {
       const int parts = (int)((v[k] + b.share.chunk - 1) / b.share.chunk);
       const int slot = atomicAdd(&b.share.counts[1], 1);
       const int at = atomicAdd(&b.share.counts[0], parts - 1);
@@ -112,7 +120,6 @@ __global__ void __launch_bounds__(kScanT) bin_chunk_out_kernel(BinBufs b, int64_
 __global__ void __launch_bounds__(1024) bin_part_scan_kernel(BinBufs b, int64_t m) {
   __shared__ int64_t part[1024];
   const int tid = threadIdx.x;
-  if (b.share.chunk > 0 && tid < 2) b.share.counts[tid] = 0;
   const int64_t per = (m + 1023) / 1024;
   const int64_t lo = tid * per, hi = (lo + per < m) ? lo + per : m;
   int64_t s = 0;
@@ -124,6 +131,10 @@ __global__ void __launch_bounds__(1024) bin_part_scan_kernel(BinBufs b, int64_t 
     __syncthreads();
     part[tid] += v;
     __syncthreads();
+  }
+  if (b.share.chunk > 0 && tid == 0) {
+    *b.share.line = share_line(part[1023], b.share.counts[2], b.share.chunk);
+    b.share.counts[0] = b.share.counts[1] = b.share.counts[2] = 0;
   }
   int64_t run = part[tid] - s;  // exclusive prefix of this thread's chunk
   for (int64_t i = lo; i < hi; ++i) {
