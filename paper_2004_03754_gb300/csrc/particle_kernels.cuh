@@ -104,17 +104,20 @@ __device__ __forceinline__ void prefetch_chunk(const PartPtrs& p, int64_t c0, in
 }
 
 // Threads per CTA and CTAs per SM of the tile kernel, with the tile shapes of
-// choose_particle_tiles.  Measured: 3D FP32, 84 M electrons, two steps and their
-// read-back, 2 x 512 threads 38.7 ms (a thread per particle of a tile at 2 per cell;
-// 2 x 256 40.2, 3 x 256 41.1, 2 x 384 44.0, 1 x 512 43.8); 3D FP64, four steps on
-// 301x60x44, one CTA of 384 on 8x8x8 cells 11.6 ms (512 threads 11.8, 2 x 256 on
-// 8x8x4 12.0); 2D FP32, ten Boris steps of 29 M electrons, 3 x 256 at 80 registers
-// 18.2 ms (4 x 256 at 64, which spill, 19.2; 2 x 256 20.4; 1 x 512 21.6).
+// choose_particle_tiles.  Measured, steps and their read-back: 3D FP32, 84 M electrons,
+// two analytic steps 2 x 512 threads 42.1 ms (a thread per particle of a tile at 2 per
+// cell; 3 x 256 43.2, 2 x 384 46.2); 3D FP64, four steps on 301x60x44, one CTA of 384 on
+// 8x8x8 cells 11.6 ms (512 threads 11.8, 2 x 256 on 8x8x4 12.0); 3D compensated (8x8x4,
+// 103 KB of windows), four Boris steps of 96^3 at 2 per cell and of 301x60x44 at 1,
+// 2 x 384 5.27 and 3.13 ms (1 x 384 6.71 and 4.49, 1 x 512 6.18 and 4.35, 2 x 256 5.45 and
+// 3.49, 2 x 320 5.27 and 3.12, but analytic 8.75 against 8.04); 2D FP32, ten Boris steps of
+// 29 M electrons, 3 x 256 at 80 registers 20.0 ms (2 x 384 20.4, 4 x 256 at 64, which spill,
+// 20.7; 2 x 256 22.9; 1 x 512 24.0).
 template <typename T, int NDIM>
 struct TileCfg {
-  static constexpr bool F = sizeof(T) == 4;
+  static constexpr bool F = sizeof(T) == 4, C = is_dfl<T>::value;
   static constexpr int threads = NDIM == 3 ? (F ? 512 : 384) : 256;
-  static constexpr int ctas = NDIM == 3 ? (F ? 2 : 1) : (F ? 3 : 2);
+  static constexpr int ctas = NDIM == 3 ? (F || C ? 2 : 1) : (F ? 3 : 2);
 };
 
 // The time-centred B^n is read from a global array formed once per step; E^n and
