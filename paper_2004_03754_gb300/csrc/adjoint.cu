@@ -660,6 +660,7 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
     PCK(pic_load_particles(c, n, x, u, w ? w : w0.data(), -1.0, 0));
   }
   const double qm = c->qm;
+  const int64_t done = c->steps_done;
   auto state = [&](int64_t k, double** f) {   // field state k of the segment in memory
     for (int m = 0; m < 6; ++m) f[m] = segF.at(k, m);
   };
@@ -804,6 +805,7 @@ pic_status laser_energy_adjoint(pic_ctx* c, const pic_laser* laser, int64_t n, c
   // leave the state at the end of the forward run
   if (c->spec || c->mw_start >= 0) PCK(load_fields(c, finF));
   PCK(pic_load_particles(c, n, xend, uend, wdev, qm, 1));
+  c->steps_done = done + 2 * nsteps;   // each step forward and once more for the reverse pass
   return pic_sync(c);
 }
 
