@@ -230,6 +230,7 @@ __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::c
   __syncthreads();
   float S = 1.0f, L = 1.0f;
   int eS = 0, l64 = 0;
+  bool finite;
   {
     unsigned long long wm = 0ull;
     for (int k = 0; k < nwarp; ++k) wm = max(wm, wmax_warp[k]);
@@ -238,6 +239,7 @@ __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::c
     // magnitude: the node sums of the quadratic spline have slope <= 1) times a
     // time-averaged shape weight (<= 1), so at most |w| |v_d| < |w|; the 2D
     // out-of-plane term is w v3 times a path-averaged weight product (<= 1)
+    finite = wm < 0x7ff0000000000000ull;
     if constexpr (F64) fix64_scales(tend - tbeg, __longlong_as_double((long long)wm), eS, l64);
     else fix_scales(tend - tbeg, narrow_signed(__longlong_as_double((long long)wm)) * 1.001f, S, L);
   }
@@ -259,10 +261,11 @@ __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::c
     else acc[c] = FixAcc{sJh + c * nW, sJl + c * nW, W[0], W[0] * W[1], S, L};
   }
   const float invS = 1.0f / S, invSL = 1.0f / (S * L);   // powers of two: exact
-  // FP64 limb weights 2^-eS, 2^-(eS + l), 2^-(eS + 2l), from the exponent bits
+  // FP64 limb weights 2^-eS, 2^-(eS + l), 2^-(eS + 2l), from the exponent bits; with an
+  // infinite or NaN weight in the tile the integers mean nothing and its current is NaN
   auto pow2 = [](int e) { return __longlong_as_double((long long)(uint64_t)(1023 + e) << 52); };
-  const double i0 = F64 ? pow2(-eS) : 0.0, i1 = F64 ? pow2(-eS - l64) : 0.0,
-               i2 = F64 ? pow2(-eS - 2 * l64) : 0.0;
+  const double i0 = F64 ? (finite ? pow2(-eS) : __longlong_as_double(0x7ff8000000000000ll)) : 0.0,
+               i1 = F64 ? pow2(-eS - l64) : 0.0, i2 = F64 ? pow2(-eS - 2 * l64) : 0.0;
   // value of window node q of component c
   auto jval = [&](int c, int q) -> D {
     if constexpr (F64) return fix64_decode(sJh[c * nW + q], sJl[c * nW + q], sJc[c * nW + q], i0, i1, i2);
