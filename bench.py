@@ -222,9 +222,9 @@ def run_gpu(args):
     value = whole_job_rate(npart, steps, world, ms_local)
     cells_s = whole_job_rate(ncell, steps, world, ms_local)
     t = mixed["timing"]
-    # roofline of the dominant kernel (particles), 88 algorithmic bytes per push
-    # against HBM.  What binds it is warp issue (74 % of the slots) and the shared-memory
-    # pipe (61 %): the push runs in FP32 pairs, so the FP64 pipe holds little work.
+    # HBM view of the dominant kernel (particles), 88 algorithmic bytes per push.  The
+    # kernel is bound by instructions (issue, FP64 and shared-memory pipes; counters in
+    # profiles/particle_kernels_counters.md)
     part_ms = t.ms_particles / steps
     alg_bytes = 88.0 * npart
     peak, peak_kind = measured_peaks()
@@ -324,7 +324,7 @@ def run_gpu(args):
     line = {
         "metric": METRIC, "value": value, "unit": METRIC, "n_gpus": world, "steps": steps,
         "warmup": warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "f32 fields + f64 pusher", "data": "synthetic",
+        "vs_baseline": None, "dtype": "f32 fields + f64 pusher (rotation in f32 pairs)", "data": "synthetic",
         "config": {"workload": WORKLOAD, "cells": list(n), "particles": npart,
                    "ppc": 8, "precision": "mixed", "parallelism": "replicas" if world > 1 else "single",
                    "l2": "inputs larger than L2 (particle state 1.4 GB)"},
@@ -332,12 +332,11 @@ def run_gpu(args):
         "kernel_ms_per_step": {"rebin": t.ms_rebin / steps, "particles": part_ms,
                                "stragglers": t.ms_stragglers / steps,
                                "correction": t.ms_correction / steps, "fields": fld_ms},
-        "roofline": {"bound": "hbm", "kernel": "particle_kernel<float,2>",
+        "roofline": {"bound": "alu", "view": "hbm bytes", "kernel": "particle_kernel<float,2>",
                      "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "peak_kind": peak_kind,
                      "alg_bytes_per_launch": alg_bytes, "traffic": None,
-                     "traffic_source": "not captured for the bench workload",
-                     "binding": "warp issue 74 %, shared-memory pipe 61 % (ncu, 2048x512 case)"},
+                     "traffic_source": "not captured for the bench workload"},
         "field_kernel_roofline": {"bound": "hbm", "kernel": "faraday_rows_kernel + ampere_rows_kernel",
                                   "achieved": fld_gbs, "peak": peak, "unit": "GB/s",
                                   "frac": fld_gbs / peak, "alg_bytes_per_cell": 60,

@@ -133,7 +133,8 @@ typedef struct {
   int correction_active;   /* 1 when C^B != e_1 (x1 current correction runs) */
   double cfl_lhs;          /* max over k of the left side of Eq. (21) */
   double cfl_sufficient_dt;/* bound of Eq. (22) */
-  int kernels_per_step;    /* kernel launches of one pic_step(ctx, 1) */
+  int kernels_per_step;    /* kernel launches of one pic_step(ctx, 1), without re-binning
+                              and the pass over particles outside their windows */
 } pic_info;
 
 /* Create a context: validates the grid, copies the coefficients, checks the

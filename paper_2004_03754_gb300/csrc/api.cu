@@ -535,8 +535,10 @@ pic_status pic_init(const pic_grid* grid, double dt, const pic_coeffs* coeffs, v
   c->corr = false;
   for (int j = 0; j < c->M; ++j)
     if (c->cB[j] != (j == 0 ? 1.0 : 0.0)) c->corr = true;
-  // field tiles: wide along x1 to amortise the 2M-1 halo of the x1 stencils
-  // (shapes from a sweep on the 4096x1024 and 512x128x128 grids)
+  // Shapes of the fused field kernels, which run on large 2D FP32 grids without
+  // particles and where the caller chose a shape (field_step_fused); the figures below
+  // compare them with one another.  Tiles wide along x1 to amortise the 2M-1 halo of
+  // the x1 stencils (shapes from a sweep on the 4096x1024 and 512x128x128 grids).
   c->ftile.threads = 256;
   c->ftile.staging = 0;
   // 2D rows (J read into registers, not staged): FP32 224 columns x 4 warps x 3

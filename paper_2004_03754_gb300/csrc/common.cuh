@@ -175,7 +175,10 @@ inline PartArgs part_args(double qm, double dt, int pusher, int64_t np) {
 // Few enough particles to take a warp each instead of tiles (FP64 fields; FP32 currents
 // keep their windows, whose sums are rounded once): 512x128 cells with one electron, 20
 // steps 0.889 -> 0.731 ms; the adjoint of 64 electrons, 1024x256, 74.6 -> 67.8 ms.  256
-// warps, two per SM, end before a tile has staged its window.
+// warps, two per SM, end before a tile has staged its window.  Their currents meet in
+// FP64 atomics on the grid, in any order: electrons that share nodes leave last-bit
+// differences from run to run, as electrons of neighbouring tiles always did; within
+// one tile's integer window there were none.
 __host__ __device__ inline bool particles_sparse(bool f64, int64_t np) { return f64 && np <= 256; }
 
 // Crowded tiles: a tile of more than `line` particles is shared by several CTAs of up to

@@ -31,7 +31,7 @@ struct pic_ctx {
   void* fb[2][3] = {{nullptr}};
   void* fj[3] = {nullptr};
   void* jtmp = nullptr;
-  void* bbar[3] = {nullptr};  // time-centred B (3D particle step)
+  void* bbar[3] = {nullptr};  // time-centred B (particle step, 2D and 3D)
   double* scratch = nullptr;  // FP64 ncell, for load/read conversions
   double* rbuf = nullptr;     // particle read-back in the original order (grown on demand)
   int64_t rbuf_n = 0;

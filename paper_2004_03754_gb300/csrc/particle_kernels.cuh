@@ -128,7 +128,8 @@ struct TileCfg {
 // nodes of E, B and 1872 of the current), so the window's handling counts as much as
 // the particles': copied and flushed value by value it took half the kernel's
 // instructions (84 M electrons, two steps and their read-back 62.8 -> 38.7 ms; 2D,
-// 29 M electrons, ten steps 23.7 -> 19.1 ms).
+// 29 M electrons, ten steps 23.7 -> 19.1 ms; both with a cheaper, less accurate push
+// than now, 42.1 and 20.0 ms).
 template <typename T, int NDIM, int PUSH, bool GAIN>
 __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::ctas)
     particle_kernel(FieldPtrs<T> f, BbarPtrs<T> bg, PartPtrs p, GridArgs g, StencilArgs<T> s,
