@@ -223,8 +223,7 @@ def run_gpu(args):
     cells_s = whole_job_rate(ncell, steps, world, ms_local)
     t = mixed["timing"]
     # HBM view of the dominant kernel (particles), 88 algorithmic bytes per push.  The
-    # kernel is bound by instructions (issue, FP64 and shared-memory pipes; counters in
-    # profiles/particle_kernels_counters.md)
+    # kernel is bound by instructions (issue, FP64 and shared-memory pipes)
     part_ms = t.ms_particles / steps
     alg_bytes = 88.0 * npart
     peak, peak_kind = measured_peaks()

@@ -10,8 +10,8 @@
 //                         arguments of the exponential are below 1/8.
 // The electric kicks, s L U, the residual of the proper time, gamma and the move
 // (dt/gamma) u stay in FP64.  Every other particle, infinities, NaN and momenta past
-// 2^40 among them, takes the FP64 push.  34 -> 22 FP64 instructions per 2D Boris push
-// against the FP64 form with its cells; 3D analytic 153 -> 66.
+// 2^40 (analytic 2^30) among them, takes the FP64 push.  FP64 instructions per push,
+// against the FP64 form: 2D Boris 34 -> 22, 3D analytic 153 -> 66.
 //
 // Error against 64 bits (113-bit reference on the device, 5e5 electrons in pulses of
 // a0 = 1 to 100 with plasma fields, at rest to gamma = 600): |du|/|u| root mean square
@@ -215,7 +215,7 @@ PIC_HD void pr_apply(const float eb[6], float s, const dfl V[4], dfl o[4]) {
 PIC_HD bool analytic_push_weak(double D, const float eb[6], double u[3]) {
   const uint32_t m0 = mag_word(u[0]), m1 = mag_word(u[1]), m2 = mag_word(u[2]);
   const uint32_t m01 = m0 > m1 ? m0 : m1, mm = m01 > m2 ? m01 : m2;
-  bool inside = mm < mag_word_of(40);
+  bool inside = mm < mag_word_of(30);   // (with |D| > 2^-20: s^2 and its low part normal)
   const double x0 = 1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
   const double ig0 = rsqrt_nr(x0), g0 = x0 * ig0;
   double E[6], LU[4];
