@@ -7,21 +7,21 @@
 // fields leaves less accurate (one Newton step per reciprocal, 2^-44):
 //   Boris, Higuera-Cary   the rotation about B, while |t| = |h B|/gamma < 1/4;
 //   analytic              what L^2 and higher powers add to U + s L U, while the
-//                         arguments of the exponential are below 1/8.
+//                         arguments of the exponential are below 1/16.
 // The electric kicks, s L U, the residual of the proper time, gamma and the move
 // (dt/gamma) u stay in FP64.  Every other particle, infinities, NaN and momenta past
 // 2^40 (analytic 2^30) among them, takes the FP64 push.  FP64 instructions per push,
-// against the FP64 form: 2D Boris 34 -> 22, 3D analytic 153 -> 66.
+// against the FP64 form: 2D Boris 34 -> 22, 3D analytic 153 -> 68.
 //
 // Error against 64 bits (113-bit reference on the device, 5e5 electrons in pulses of
 // a0 = 1 to 100 with plasma fields, at rest to gamma = 600): |du|/|u| root mean square
 // and 99th percentile, the FP64 form before the arrow
 //   Boris 3.8e-16 -> 3.4e-16, 1.3e-15 -> 1.1e-15;  Higuera-Cary 2.0e-15 -> 3.3e-16,
-//   6.2e-15 -> 1.2e-15;  analytic 1.1e-16 -> 8.1e-17, 2.5e-16 -> 1.8e-16;
+//   6.2e-15 -> 1.2e-15;  analytic 1.1e-16 -> 7.4e-17, 2.5e-16 -> 1.7e-16;
 // the move 3.2e-15 dt in all (the reciprocal's one Newton step).
 // Measured: 2D Boris, 29.4 M electrons, ten steps and their read-back, all FP64 rotation
 // and cells 24.2 -> 20.2 ms; 2D Higuera-Cary, 1.4 M, twelve steps 2.80 -> 2.24 ms; 3D
-// analytic, 84 M, two steps 54.8 -> 42.1 ms.
+// analytic, 84 M, two steps 54.8 -> 42.8 ms.
 //
 // Products feeding a TwoSum are rounded on their own (mul_rn); sums written
 // plainly hold no product, so no contraction can break them.
@@ -202,16 +202,18 @@ PIC_HD void pr_apply(const float eb[6], float s, const dfl V[4], dfl o[4]) {
   for (int d = 0; d < 4; ++d) o[d] = pr_norm(pr_mulf(o[d], s));
 }
 
-// The analytic push (analytic_series.cuh) while L s is small, |s|^2 (E^2 + B^2) < 2^-6: U(s) =
+// The analytic push (analytic_series.cuh) while L s is small, |s|^2 (E^2 + B^2) < 2^-8: U(s) =
 // U + s L U + R(s) in s = (q/m) tau with the raw fields; s L U, of size |L s| |U|, in
 // FP64 and R, of size |L s|^2 |U|/2, in pairs, so that R's rounding, 2^-48 of it, stays
-// below FP64's.  With b_k = s^k L^k U, A = S1 s^2, Q = S2 s^4 (|A| < 2^-6, Q < 2^-14) and
-// p_1 = 1, p_2 = A, p_3 = A^2 + Q, p_4 = A^3 + 2 A Q, s_a = sum_n p_n/(2n + a)!,
+// below FP64's.  With b_k = s^k L^k U, A = S1 s^2, Q = S2 s^4 (|A| < 2^-8, Q < 2^-18) and
+// p_1 = 1, p_2 = A, p_{n+1} = A p_n + Q p_{n-1}, s_a = sum_n p_n/(2n + a)!,
 //   R = s_0 b_2 + s_1 b_3 + Q s_2 U + Q s_3 b_1,
 //   F(s) = s [gamma + b_1/2 + s_1 b_2 + s_2 b_3 + Q s_3 gamma + Q s_4 b_1] (time components)
-// is q/m times the lab time.  An FP32 Newton gives s to about 2^-22, the FP64 residual
+// is q/m times the lab time.  An FP32 Newton gives s to about 2^-23, the FP64 residual
 // F(s) - (q/m) dt the rest, delta, which moves s in the FP64 term and R to second order.
-// False outside, with u unchanged.
+// The line: for electrons at rest R is B s/2 of u, so the pairs' share grows with |L s|;
+// root mean square error of |u| for |L s| from 2^-5 to 2^-4 1.2e-16 (FP64 form 1.4e-16),
+// up to 2^-3 it would be 1.8e-16.  False outside, with u unchanged.
 PIC_HD bool analytic_push_weak(double D, const float eb[6], double u[3]) {
   const uint32_t m0 = mag_word(u[0]), m1 = mag_word(u[1]), m2 = mag_word(u[2]);
   const uint32_t m01 = m0 > m1 ? m0 : m1, mm = m01 > m2 ? m01 : m2;
@@ -227,12 +229,13 @@ PIC_HD bool analytic_push_weak(double D, const float eb[6], double u[3]) {
     const int a = (d + 1) % 3, b = (d + 2) % 3;
     LU[d + 1] = fma(g0, E[d], fma(u[a], E[3 + b], -(u[b] * E[3 + a])));
   }
+  const double sd = D * ig0;
   const float Df = narrow_sat(D), ig = narrow_sat(ig0);
   const dfl ee = pr_sum3(pr_mulff(eb[0], eb[0]), pr_mulff(eb[1], eb[1]), pr_mulff(eb[2], eb[2]));
   const dfl bb = pr_sum3(pr_mulff(eb[3], eb[3]), pr_mulff(eb[4], eb[4]), pr_mulff(eb[5], eb[5]));
   const dfl dot = pr_sum3(pr_mulff(eb[0], eb[3]), pr_mulff(eb[1], eb[4]), pr_mulff(eb[2], eb[5]));
-  const float sa = Df * ig;
-  inside = inside && sa * sa * (ee.hi + bb.hi) < 0.015625f && fabsf(Df) > 0x1p-20f && fabsf(Df) < 0x1p20f;
+  const float sa = narrow_sat(sd);
+  inside = inside && sa * sa * (ee.hi + bb.hi) < 0.00390625f && fabsf(Df) > 0x1p-20f && fabsf(Df) < 0x1p20f;
   if (!inside) return false;                        // (also NaN)
   dfl V0[4], b1[4], b2[4], b3[4];
   V0[0] = pr_split(g0);
@@ -241,9 +244,12 @@ PIC_HD bool analytic_push_weak(double D, const float eb[6], double u[3]) {
   dfl W1[4];
 #pragma unroll
   for (int d = 0; d < 4; ++d) W1[d] = pr_split(LU[d]);
-  // s in FP32: Newton on s (1 + s (p/2 + s (r/6 + s t/24))) = D/gamma, L^k U in FP32
+  // s in FP32: Newton on s (1 + s (p + s (r + s (t + s v)))) = D/gamma, the terms of L^k U in
+  // FP32 (L^4 = S1 L^2 + S2), the right side with its low part, so that s is good to its
+  // last place
   float s = sa;
   {
+    const float sl = narrow_signed(sd - widen(sa));
     float w[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -253,9 +259,10 @@ PIC_HD bool analytic_push_weak(double D, const float eb[6], double u[3]) {
     const float p = 0.5f * (W1[0].hi * ig);
     const float r = 0.16666667f * (fmaf(eb[0], W1[1].hi, fmaf(eb[1], W1[2].hi, eb[2] * W1[3].hi)) * ig);
     const float t = 0.041666668f * (fmaf(eb[0], w[0], fmaf(eb[1], w[1], eb[2] * w[2])) * ig);
+    const float v = fmaf(ee.hi - bb.hi, 0.05f * r, 0.0083333333f * (dot.hi * dot.hi));
 #pragma unroll
     for (int it = 0; it < 3; ++it) {
-      const float F = fmaf(s * s, fmaf(s, fmaf(s, t, r), p), s - sa);
+      const float F = fmaf(s * s, fmaf(s, fmaf(s, fmaf(s, v, t), r), p), (s - sa) - sl);
       const float G = s * fmaf(s, fmaf(s, 4.0f * t, 3.0f * r), 2.0f * p);   // dF/ds - 1, small
       s = fmaf(-F, fmaf(G, G, 1.0f - G), s);
     }
@@ -266,10 +273,12 @@ PIC_HD bool analytic_push_weak(double D, const float eb[6], double u[3]) {
   pr_apply(eb, s, b2, b3);
   const dfl z = pr_mulff(s, s);
   const dfl A = pr_norm(pr_mul(pr_add(ee, pr_neg(bb)), z)), dz = pr_norm(pr_mul(dot, z)), Q = pr_norm(pr_sqr(dz));
-  const float p3 = fmaf(A.hi, A.hi, Q.hi), p4 = A.hi * fmaf(A.hi, A.hi, 2.0f * Q.hi);
-  // 1/3!, 1/4!, 1/5! as pairs
-  const dfl i6(PIC_AS.h3[0], PIC_AS.l3[0]), i24(PIC_AS.h2[1], PIC_AS.l2[1]), i120(PIC_AS.h3[1], PIC_AS.l3[1]);
-  const dfl s0 = pr_sum3(dfl(0.5f, 0.0f), pr_mul(A, i24), dfl(fmaf(p4, PIC_AS.h2[3], p3 * PIC_AS.h2[2]), 0.0f));
+  const dfl P3 = pr_add(pr_sqr(A), Q);
+  const float p3 = P3.hi, p4 = A.hi * fmaf(A.hi, A.hi, 2.0f * Q.hi);
+  // 1/3!, 1/4!, 1/5!, 1/6! as pairs
+  const dfl i6(PIC_AS.h3[0], PIC_AS.l3[0]), i24(PIC_AS.h2[1], PIC_AS.l2[1]), i120(PIC_AS.h3[1], PIC_AS.l3[1]),
+            i720(PIC_AS.h2[2], PIC_AS.l2[2]);
+  const dfl s0 = pr_sum3(dfl(0.5f, 0.0f), pr_mul(A, i24), pr_add_raw(pr_mul(P3, i720), dfl(p4 * PIC_AS.h2[3], 0.0f)));
   const dfl s1 = pr_sum3(i6, pr_mul(A, i120), dfl(fmaf(p4, PIC_AS.h3[3], p3 * PIC_AS.h3[2]), 0.0f));
   const dfl s2 = pr_add(i24, dfl(fmaf(p3, PIC_AS.h2[3], A.hi * PIC_AS.h2[2]), 0.0f));
   const dfl q3 = pr_norm(pr_mul(Q, pr_add(i120, dfl(A.hi * PIC_AS.h3[2], 0.0f))));
@@ -284,9 +293,9 @@ PIC_HD bool analytic_push_weak(double D, const float eb[6], double u[3]) {
   const float d1f = narrow_signed(d1), e = d1f * seed_rcp(s);   // delta, delta/s
   // second order of Newton: -(gamma'/2 gamma) delta^2
   const float d2 = -0.5f * narrow_signed(rg) * (b1[0].hi + fmaf(0.5f, b3[0].hi, b2[0].hi)) * (e * d1f);
-  if (!(fabsf(e) <= 0x1p-20f)) return false;         // not settled, NaN
+  if (!(fabsf(e) <= 0x1p-21f)) return false;         // not settled, NaN
   const double sn = s64 + (d1 + widen(d2));
-  // R(s + delta) = R + delta L (s L U + R) + (delta^2/2) L^2 U
+  // R(s + delta) = R + delta L (s L U + R) + (delta^2/2) L^2 (U + s L U)
   dfl R[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d)
@@ -296,7 +305,7 @@ PIC_HD bool analytic_push_weak(double D, const float eb[6], double u[3]) {
   for (int d = 0; d < 3; ++d) {
     const int a = (d + 1) % 3, b = (d + 2) % 3;
     const float T = s * fmaf(Rg, eb[d], fmaf(R[a].hi, eb[3 + b], -(R[b].hi * eb[3 + a])));
-    const float dR = e * (fmaf(0.5f * e, b2[d + 1].hi, b2[d + 1].hi) + T);
+    const float dR = e * (fmaf(0.5f * e, b2[d + 1].hi + b3[d + 1].hi, b2[d + 1].hi) + T);
     u[d] = fma(sn, LU[d + 1], u[d] + pr_join(pr_add(R[d], dfl(dR, 0.0f))));
   }
   return true;

@@ -105,8 +105,8 @@ __device__ __forceinline__ void prefetch_chunk(const PartPtrs& p, int64_t c0, in
 
 // Threads per CTA and CTAs per SM of the tile kernel, with the tile shapes of
 // choose_particle_tiles.  Measured, steps and their read-back: 3D FP32, 84 M electrons,
-// two analytic steps 2 x 512 threads 42.1 ms (a thread per particle of a tile at 2 per
-// cell; 3 x 256 43.2, 2 x 384 46.2); 3D FP64, four steps on 301x60x44, one CTA of 384 on
+// two analytic steps 2 x 512 threads 42.8 ms (a thread per particle of a tile at 2 per
+// cell; 3 x 256 44.6, 2 x 384 47.8); 3D FP64, four steps on 301x60x44, one CTA of 384 on
 // 8x8x8 cells 11.6 ms (512 threads 11.8, 2 x 256 on 8x8x4 12.0); 3D compensated (8x8x4,
 // 103 KB of windows), four Boris steps of 96^3 at 2 per cell and of 301x60x44 at 1,
 // 2 x 384 5.27 and 3.13 ms (1 x 384 6.71 and 4.49, 1 x 512 6.18 and 4.35, 2 x 256 5.45 and
@@ -129,7 +129,7 @@ struct TileCfg {
 // the particles': copied and flushed value by value it took half the kernel's
 // instructions (84 M electrons, two steps and their read-back 62.8 -> 38.7 ms; 2D,
 // 29 M electrons, ten steps 23.7 -> 19.1 ms; both with a cheaper, less accurate push
-// than now, 42.1 and 20.0 ms).
+// than now, 42.8 and 20.0 ms).
 template <typename T, int NDIM, int PUSH, bool GAIN>
 __global__ void __launch_bounds__(TileCfg<T, NDIM>::threads, TileCfg<T, NDIM>::ctas)
     particle_kernel(FieldPtrs<T> f, BbarPtrs<T> bg, PartPtrs p, GridArgs g, StencilArgs<T> s,

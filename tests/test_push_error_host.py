@@ -62,10 +62,7 @@ def _electrons(r):
     return dt, fields(last * dt).astype(np.float32).astype(np.float64), u
 
 
-@pytest.mark.parametrize("r", [0.5, 0.25])
-@pytest.mark.parametrize("kind", [0, 1, 2], ids=["boris", "analytic", "hc"])
-def test_error_is_no_larger(harness, tmp_path, kind, r):
-    dt, F, u = _electrons(r)
+def _run(harness, tmp_path, kind, dt, F, u):
     rec = np.empty(N, dtype=[("kind", "<i4"), ("v", "<f8", 11)])
     rec["kind"] = kind
     rec["v"] = np.concatenate([np.full((1, N), -1.0), np.full((1, N), dt), F, u]).T
@@ -74,8 +71,35 @@ def test_error_is_no_larger(harness, tmp_path, kind, r):
         f.write(struct.pack("<i", N))
         f.write(rec.tobytes())
     subprocess.check_call([harness, str(fin), str(fout)])
-    e = np.fromfile(fout, dtype="<f8").reshape(N, 4)
+    return np.fromfile(fout, dtype="<f8").reshape(N, 4)
+
+
+@pytest.mark.parametrize("r", [0.5, 0.25])
+@pytest.mark.parametrize("kind", [0, 1, 2], ids=["boris", "analytic", "hc"])
+def test_error_is_no_larger(harness, tmp_path, kind, r):
+    dt, F, u = _electrons(r)
+    e = _run(harness, tmp_path, kind, dt, F, u)
     for mine, fp64 in ((e[:, 0], e[:, 1]), (e[:, 2], e[:, 3])):
         assert np.sqrt(np.mean(mine ** 2)) <= 1.02 * np.sqrt(np.mean(fp64 ** 2))
         assert np.quantile(mine, 0.99) <= 1.02 * np.quantile(fp64, 0.99)
         assert np.median(mine) <= 1.02 * np.median(fp64)
+
+
+@pytest.mark.parametrize("cold", [True, False])
+@pytest.mark.parametrize("kind", [0, 1, 2], ids=["boris", "analytic", "hc"])
+def test_error_in_the_pairs_range(harness, tmp_path, kind, cold):
+    # across the lines past which the FP64 push takes over: |s|^2 (E^2 + B^2) to 2^-6, weak
+    # and strong shares of E and B, electrons at rest (|u| error against their new u, so
+    # the fields' share is as large as it gets) and hot ones
+    rng = np.random.Generator(np.random.PCG64(6))
+    dt = 2 * math.pi / 64
+    u = np.zeros((3, N)) if cold else rng.normal(0, 1, (3, N)) * 10.0 ** rng.uniform(-3, 3, N)
+    gam = np.sqrt(1 + (u * u).sum(0))
+    F = rng.normal(0, 1, (6, N))
+    F[:3] *= 10.0 ** rng.uniform(-4, 0, N)
+    F *= gam / dt * 2.0 ** rng.uniform(-8, -3, N) / np.sqrt((F * F).sum(0))
+    e = _run(harness, tmp_path, kind, dt, F.astype(np.float32).astype(np.float64), u)
+    for q in (0.5, 0.99, 0.999):
+        # (a rest of rounding of the pairs, 2^-48 of a change of u of up to a tenth)
+        assert np.quantile(e[:, 0], q) <= max(1.02 * np.quantile(e[:, 1], q), 2.0 ** -48 / 10 * 5), q
+        assert np.quantile(e[:, 2], q) <= 1.02 * np.quantile(e[:, 3], q), q
